@@ -216,7 +216,8 @@ struct lb_ctx {
     int sweep_occ6 = 0;              // its occupancy variant
     int tma_tile = 0;                // tile shape of the tensor maps (see lb_step_tma.cu)
     int tma_tile_fixed = -1;         // LBFLUCT_TMA_TILE, else -1: the fastest for the noise mode
-    alignas(64) unsigned char tmap[2][128];
+    alignas(64) unsigned char tmap[2][128];     // per buffer: loads
+    alignas(64) unsigned char tmap_out[2][128]; // and stores
     double fbar[Q] = {};
     // parameters
     bool have_params = false;
@@ -381,8 +382,8 @@ int lb_create(int nx, int ny, int precision, uint64_t seed, double rho0, double 
         if (c->tma_tile_fixed >= tma_tile_count()) c->tma_tile_fixed = -1;
         c->tma_tile = c->tma_tile_fixed >= 0 ? c->tma_tile_fixed : tma_default_tile(LB_NOISE_LW, c->fp16);
         c->use_tma = want_tma && tensor_map_bytes() <= sizeof(c->tmap[0]) &&
-                     make_pop_tensor_map(c->pop[0], g, c->tma_tile, c->fp16, c->tmap[0]) &&
-                     make_pop_tensor_map(c->pop[1], g, c->tma_tile, c->fp16, c->tmap[1]);
+                     make_pop_tensor_maps(c->pop[0], g, c->tma_tile, c->fp16, c->tmap[0], c->tmap_out[0]) &&
+                     make_pop_tensor_maps(c->pop[1], g, c->tma_tile, c->fp16, c->tmap[1], c->tmap_out[1]);
     }
 
     // host tables in FP64 -> device
@@ -718,12 +719,13 @@ int lb_step(lb_ctx* c, int64_t nsteps) {
             const int want = (c->tma_tile_fixed >= 0 && !poly) ? c->tma_tile_fixed : tma_default_tile(kmode, c->fp16);
             if (want != c->tma_tile) {
                 // tensor maps are host-encoded descriptors passed by value: re-encode for the shape
-                if (!make_pop_tensor_map(c->pop[0], c->g, want, c->fp16, c->tmap[0]) ||
-                    !make_pop_tensor_map(c->pop[1], c->g, want, c->fp16, c->tmap[1]))
+                if (!make_pop_tensor_maps(c->pop[0], c->g, want, c->fp16, c->tmap[0], c->tmap_out[0]) ||
+                    !make_pop_tensor_maps(c->pop[1], c->g, want, c->fp16, c->tmap[1], c->tmap_out[1]))
                     return fail(c, LB_ECUDA, "tensor map encoding failed");
                 c->tma_tile = want;
             }
-            CK(c, launch_step_tma(a, c->tmap[c->cur], c->err_dev, kmode, c->tma_tile, c->fp16, c->stream, poly),
+            CK(c, launch_step_tma(a, c->sad, c->tmap[c->cur], c->tmap_out[c->cur ^ 1], c->err_dev, kmode, c->tma_tile, c->fp16,
+                                  c->stream, poly),
                "step kernel launch");
         } else
             CK(c, launch_step_simple(a, kmode, c->fp16, c->stream), "step kernel launch");

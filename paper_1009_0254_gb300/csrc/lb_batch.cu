@@ -2,10 +2,10 @@
 //
 // Replicas of equal size form a class.  A class keeps its populations replica-major in
 // one buffer pair, [replica][plane][row][column] with the single-lattice layout per replica,
-// so one 4D tensor map (x, y, plane, replica) serves the whole class.  One persistent launch
+// so one 4D tensor map (x, y, plane, replica) for loads and one for stores serve the whole class.  One persistent launch
 // of the batched TMA step kernel advances every replica of up to MAX_CLASSES classes by one
 // step: the launch's tiles are numbered class by class, replica by replica, and every CTA
-// walks its share of them through a two-stage TMA pipeline.  Each replica keeps its own
+// walks its share of them, the next tile's load and the last one's store behind a tile's collision.  Each replica keeps its own
 // Philox key (its seed), relaxation and noise factors and time offset in a device record;
 // the step counter K lives in device memory and is advanced by the last CTA of the step's
 // last launch, so a captured CUDA graph of G steps can be replayed as it is: a replica's
@@ -29,7 +29,7 @@
 
 namespace lbf {
 
-constexpr int MAX_CLASSES = 8;      // size classes per launch (kernel parameters stay < 4 KB)
+constexpr int MAX_CLASSES = 8;      // size classes per launch (about 5 KB of kernel parameters)
 
 struct ClassDesc {
     Grid g;
@@ -44,7 +44,8 @@ struct ClassDesc {
 };
 
 struct EnsParams {
-    CUtensorMap map[MAX_CLASSES][2];   // per class: map of buffer 0, of buffer 1
+    CUtensorMap map[MAX_CLASSES][2];   // per class: load map of buffer 0, of buffer 1
+    CUtensorMap out[MAX_CLASSES][2];   // per class: store map of buffer 0, of buffer 1
     ClassDesc cls[MAX_CLASSES];
     int nclass, ntiles;
     long long* kstep;                  // device step counter K
@@ -83,114 +84,125 @@ __device__ __forceinline__ TilePos locate(const EnsParams& p, int tile) {
     return t;
 }
 
+// The engine's step is the single-lattice kernel's (lb_step_tma.cu, lb_pair.cuh) plus, per tile, its
+// position and its replica's record; both bound it beside DRAM (252 to 297 instructions a node against
+// 209 and up).  512 replicas of 32^2 to 256^2, best tile: 188 us a step with scalar nodes and two
+// stages, 164 in this form; real-space correlated noise 333 and 228; 16 replicas of 1024^2 258 and 222.
 // RS: the variant that also steps replicas with real-space correlated noise (its extra path
 // raises the register count, so launches without such replicas use the lean variant)
 template <int TX, int TY, int NT, bool RS>
-__global__ void __launch_bounds__(NT, RS ? 1024 / NT : 0) step_ensemble_kernel(const __grid_constant__ EnsParams p) {
+__global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_ensemble_kernel(const __grid_constant__ EnsParams p) {
     using TT = TmaTile<TX, TY, float>;
+    using M = PairMap<TX, TY, NT>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    float* smem = reinterpret_cast<float*>(smem_raw);
-    float* R = reinterpret_cast<float*>(smem_raw + 2 * TT::STAGE_BYTES);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(R + TT::RW * TT::RH);
+    float* S = reinterpret_cast<float*>(smem_raw);
+    float* out = reinterpret_cast<float*>(smem_raw + TT::OUT);
+    float* R = reinterpret_cast<float*>(smem_raw + TT::RHO);
+    const uint32_t bar = smem_u32(smem_raw + TT::BAR);
+    unsigned char* xch = smem_raw + TT::SMEM_BYTES;     // RS: StencilTile
     __shared__ TileArgsOf<RS> sargs;    // the record of the current tile
-    __shared__ int smode;
     const int tid = threadIdx.x;
-    const long long K = __ldcg(p.kstep);
-    const int par = (int)(K & 1);
     const int ntiles = p.ntiles;
 
     if (tid == 0) {
-        mbar_init(smem_u32(&mbar[0]), 1);
-        mbar_init(smem_u32(&mbar[1]), 1);
+        mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    const long long K = __ldcg(p.kstep);
+    const int par = (int)(K & 1);
 
-    auto issue = [&](int tile, int s) {
-        const TilePos tp = locate<TX, TY>(p, tile);
+    auto load = [&](const TilePos& tp) {
         const CUtensorMap* map = &p.map[tp.c][par];
         const int gx = p.cls[tp.c].g.gx;
-        const uint32_t bar = smem_u32(&mbar[s]);
         mbar_expect_tx(bar, TT::TX_BYTES);
-        float* st = smem + s * TT::STAGE;
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            tma_load_4d(smem_u32(st + i * TT::PS), map, tp.x0 - TT::XO + gx, tp.y0 - 1 - kCYt[i] + GY, i, tp.rep,
-                        bar);
+            tma_load_4d(smem_u32(S + i * TT::PS), map, tp.x0 - TT::XO + gx, tp.y0 - 1 - kCYt[i] + GY, i, tp.rep, bar);
+    };
+    auto store = [&](const TilePos& tp) {
+        if (tile_direct<TX, float>(p.cls[tp.c].g, tp.x0)) return;
+        tma_store_4d(&p.out[tp.c][par ^ 1], smem_u32(out), tp.x0, tp.y0, 0, tp.rep);
+        tma_store_commit();
     };
 
+    // the positions of the tiles of even and odd turns: located once, by the thread that loads them
+    __shared__ TilePos pos[2];
     const int first = blockIdx.x;
-    if (tid == 0) {
-        if (first < ntiles) issue(first, 0);
-        if (first + (int)gridDim.x < ntiles) issue(first + gridDim.x, 1);
+    if (tid == 0 && first < ntiles) {
+        pos[0] = locate<TX, TY>(p, first);
+        load(pos[0]);
     }
-    int k = 0;
+    uint32_t k = 0;
     for (int tile = first; tile < ntiles; tile += gridDim.x, ++k) {
-        const int s = k & 1;
-        const TilePos tp = locate<TX, TY>(p, tile);
-        const bool ok = mbar_wait_bounded(smem_u32(&mbar[s]), (uint32_t)((k >> 1) & 1));
+        // the next tile is located while this one's populations are in flight
+        const int tn = tile + (int)gridDim.x;
+        TilePos next;
+        if (tid == 0 && tn < ntiles) next = locate<TX, TY>(p, tn);
+        const bool ok = mbar_wait_bounded(bar, k & 1u);
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 atomicExch(p.err, 1);
                 // give the loads still in flight into this CTA's shared memory a bounded
                 // chance to land before the CTA exits
-                mbar_wait_bounded(smem_u32(&mbar[s]), (uint32_t)((k >> 1) & 1));
-                if (tile + (int)gridDim.x < ntiles)
-                    mbar_wait_bounded(smem_u32(&mbar[s ^ 1]), (uint32_t)(((k + 1) >> 1) & 1));
+                mbar_wait_bounded(bar, k & 1u);
             }
+            k = 0;                     // nothing of this CTA is left to store
             break;
         }
+        const int s = (int)(k & 1u);
+        if (tid == 0 && k > 0) store(pos[s ^ 1]);
+        const TilePos tp = pos[s];
         const ClassDesc& d = p.cls[tp.c];
         const Grid g = d.g;
-        const float* S = smem + s * TT::STAGE;
         // the tile's replica record, to shared memory (its last readers, the previous tile's
         // collision, are past the barrier above; measured faster than a copy per thread in
         // registers, which the pulled populations need, and than loading it before the wait)
-        if (tid == 0) {
-            const RepRec* rp = p.cls[tp.c].recs + tp.rep;
-            load_tile_args(rp, K + __ldg(&rp->toff), &sargs, &smode);
-            if constexpr (RS) {
-                if (smode == 3) load_stencil_args(rp, &sargs);
-            }
+        {
+            const RepRec* rp = d.recs + tp.rep;
+            load_tile_args<RS>(rp, K + __ldg(&rp->toff), &sargs);
         }
 
-        // pulled populations stay in registers across the density barrier; the stage is
-        // refilled right after it
-        float fr[TX * TY / NT][Q];
-        tile_pull<TX, TY, NT, RS>(S, R, fr);
+        // pulled populations stay in registers across the density barrier; the next tile is
+        // loaded right after it
+        F2 fr[M::RPT][Q], z4[M::RPT], z9[M::RPT];
+        tile_pull<TX, TY, NT, false, RS>(S, R, fr);
+        if (tid == 0) tma_store_wait_read();
         __syncthreads();
-        if (tid == 0 && !(RS && smode == 3) && tile + 2 * (int)gridDim.x < ntiles) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue(tile + 2 * gridDim.x, s);
+        if (tid == 0 && tn < ntiles) {
+            fence_async_smem();
+            load(next);
+            pos[s ^ 1] = next;
         }
-        const int mode = smode;
+        const int mode = sargs.mode;        // the tile's: uniform over the CTA
         float* dst = (par ? d.buf[0] : d.buf[1]) + (long long)tp.rep * d.rstride;
         bool stepped = false;
         if constexpr (RS) {
             if (mode == 3) {
-                // real-space correlated noise: the contributions go to the consumed stage s,
-                // whose refill waits for the collision (the mode is the tile's: uniform over
-                // the CTA)
-                float2* Hs = reinterpret_cast<float2*>(smem_raw + s * TT::STAGE_BYTES);
-                tile_stencil<TX, TY, NT>(sargs, Hs, g, tp.x0, tp.y0);
+                stencil_tile<TX, TY, NT>(sargs, xch, tp.x0, tp.y0, g.nx, g.ny, z4, z9);
                 __syncthreads();
-                tile_nodes<3, TX, TY, NT>(sargs, fr, R, g, tp.x0, tp.y0, dst, nullptr, Hs);
-                __syncthreads();
-                if (tid == 0 && tile + 2 * (int)gridDim.x < ntiles) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    issue(tile + 2 * gridDim.x, s);
-                }
+                tile_collide<3, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
+                                                          z9, xch);
                 stepped = true;
             }
         }
         if (!stepped) {
             if (mode == 2)
-                tile_nodes<2, TX, TY, NT>(sargs, fr, R, g, tp.x0, tp.y0, dst, d.xi + (long long)tp.rep * g.nx * g.ny);
+                tile_collide<2, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst,
+                                                          d.xi + (long long)tp.rep * g.nx * g.ny, z4, z9, nullptr);
             else if (mode)
-                tile_nodes<1, TX, TY, NT>(sargs, fr, R, g, tp.x0, tp.y0, dst, nullptr);
+                tile_collide<1, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
+                                                          z9, nullptr);
             else
-                tile_nodes<0, TX, TY, NT>(sargs, fr, R, g, tp.x0, tp.y0, dst, nullptr);
+                tile_collide<0, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
+                                                          z9, nullptr);
         }
+        fence_async_smem();
+    }
+    __syncthreads();
+    if (tid == 0 && k > 0) {
+        store(pos[(k - 1u) & 1u]);
+        tma_store_wait();
     }
     // Every CTA read K before arriving here; the last one to arrive advances it for the
     // next step (the next launch sees it, kernel boundaries order the accesses).
@@ -344,40 +356,52 @@ static const int kBatchTiles[][3] = {{32, 16, 256}, {32, 16, 128}, {32, 8, 256},
                                      {64, 8, 256},  {64, 16, 512}, {32, 32, 512}};
 constexpr int kBatchTileCount = 7;
 
-static bool make_class_map(void* buf, const Grid& g, int R, int tile, CUtensorMap* map) {
+// load and store maps of one population buffer of a class of R replicas (make_pop_tensor_maps
+// with the replica as a fourth dimension)
+static bool make_class_maps(void* buf, const Grid& g, int R, int tile, CUtensorMap* load, CUtensorMap* store) {
     EncodeTiledFn fn = tensor_map_encoder();
     if (!fn || tile < 0 || tile >= kBatchTileCount) return false;
-    cuuint64_t dims[4] = {(cuuint64_t)g.pitch, (cuuint64_t)(g.ny + 2 * GY), (cuuint64_t)Q, (cuuint64_t)R};
     cuuint64_t strides[3] = {(cuuint64_t)g.pitch * 4, (cuuint64_t)g.plane * 4, (cuuint64_t)g.plane * 4 * Q};
-    // box: the tile plus 4 columns (16 bytes) on either side and one row above and below
-    cuuint32_t box[4] = {(cuuint32_t)(kBatchTiles[tile][0] + 8), (cuuint32_t)(kBatchTiles[tile][1] + 2), 1, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
+    cuuint64_t ldims[4] = {(cuuint64_t)g.pitch, (cuuint64_t)(g.ny + 2 * GY), (cuuint64_t)Q, (cuuint64_t)R};
+    // box: the tile plus 4 columns (16 bytes) on either side and one row above and below
+    cuuint32_t lbox[4] = {(cuuint32_t)(kBatchTiles[tile][0] + 8), (cuuint32_t)(kBatchTiles[tile][1] + 2), 1, 1};
     // 64-byte L2 promotion: a class's rows carry 128 bytes of ghost columns on either side of
     // which one 32-byte sector is ever written or read; with 256-byte promotion a box row
     // pulled whole rows of the small lattices (the 512-replica mix read 1.74x the algorithmic
     // bytes, 1.33x with 64; its 32^2 class 3.20x and 2.13x, 138 -> 112 us a step)
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, buf, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_64B,
+    if (fn(load, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, buf, ldims, strides, lbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+           CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_64B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
+        CUDA_SUCCESS)
+        return false;
+    cuuint64_t sdims[4] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)Q, (cuuint64_t)R};
+    cuuint32_t sbox[4] = {(cuuint32_t)kBatchTiles[tile][0], (cuuint32_t)kBatchTiles[tile][1], (cuuint32_t)Q, 1};
+    return fn(store, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, (float*)buf + g.at(0, 0), sdims, strides, sbox, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// dynamic shared memory of the step kernel
+template <int TX, int TY, int NT, bool RS>
+constexpr int ensemble_smem() {
+    return TmaTile<TX, TY, float>::SMEM_BYTES + (RS ? StencilTile<TX, TY, NT>::BYTES : 0);
 }
 
 // CTAs of a persistent launch: every SM filled to the occupancy the kernel allows
 template <int TX, int TY, int NT, bool RS>
 static cudaError_t ensemble_grid(int* grid) {
-    using TT = TmaTile<TX, TY, float>;
     static GridCache cache;
-    return resident_grid(step_ensemble_kernel<TX, TY, NT, RS>, NT, TT::SMEM_BYTES, cache, grid);
+    return resident_grid(step_ensemble_kernel<TX, TY, NT, RS>, NT, ensemble_smem<TX, TY, NT, RS>(), cache, grid);
 }
 
 template <int TX, int TY, int NT>
 static cudaError_t launch_ensemble_t(const EnsParams& p, cudaStream_t s) {
-    using TT = TmaTile<TX, TY, float>;
     int grid = 0;
     cudaError_t e = p.rs ? ensemble_grid<TX, TY, NT, true>(&grid) : ensemble_grid<TX, TY, NT, false>(&grid);
     if (e != cudaSuccess) return e;
     const int blocks = std::max(1, std::min(p.ntiles, grid));
-    if (p.rs) step_ensemble_kernel<TX, TY, NT, true><<<blocks, NT, TT::SMEM_BYTES, s>>>(p);
-    else step_ensemble_kernel<TX, TY, NT, false><<<blocks, NT, TT::SMEM_BYTES, s>>>(p);
+    if (p.rs) step_ensemble_kernel<TX, TY, NT, true><<<blocks, NT, ensemble_smem<TX, TY, NT, true>(), s>>>(p);
+    else step_ensemble_kernel<TX, TY, NT, false><<<blocks, NT, ensemble_smem<TX, TY, NT, false>(), s>>>(p);
     return cudaGetLastError();
 }
 
@@ -411,24 +435,22 @@ static cudaError_t prepare_ensemble_kernels() {
 }
 
 // Relaxation rates, Cholesky factors of Xi(0) (Sec. IV; the (4,9) block coupled unless
-// noise_mode is LB_NOISE_DIAG) and noise switch of one lattice's record; the key, time
-// offset and rho0/cs2 fields are left to the caller.
+// noise_mode is LB_NOISE_DIAG) and noise switch of one lattice's record; the key and the time
+// offset are left to the caller.
 void fill_rep_record(double rho0, double cs2, double kT, double kappa, double tau_s, double tau_b,
                      double tau_ghost, int noise_mode, RepRec* rec) {
+    constexpr double c = pair_scale<false>();
     double xi[81];
     lb_noise_matrix(rho0, cs2, kT, kappa, tau_s, tau_b, tau_ghost, 0.0, 0.0, xi);
     const double x44 = xi[3 * 9 + 3], x49 = noise_mode == LB_NOISE_DIAG ? 0.0 : xi[3 * 9 + 8], x99 = xi[8 * 9 + 8];
     const double L44 = std::sqrt(std::fmax(x44, 0.0));
     const double L94 = L44 > 0.0 ? x49 / L44 : 0.0;
     const double L99 = std::sqrt(std::fmax(x99 - L94 * L94, 0.0));
-    rec->kappa = (float)kappa;
-    rec->lb = (float)(-1.0 / tau_b);
-    rec->ls = (float)(-1.0 / tau_s);
-    rec->lq = rec->le = (float)(-1.0 / tau_ghost);
-    rec->L44 = (float)L44; rec->L49 = 0.0f; rec->L94 = (float)L94; rec->L99 = (float)L99;
-    rec->s5 = (float)std::sqrt(std::fmax(xi[4 * 9 + 4], 0.0));
-    rec->s6 = (float)std::sqrt(std::fmax(xi[5 * 9 + 5], 0.0));
-    rec->s7 = (float)std::sqrt(std::fmax(xi[6 * 9 + 6], 0.0));
+    const double L[4] = {L44, 0.0, L94, L99};
+    const double s3[3] = {std::sqrt(std::fmax(xi[4 * 9 + 4], 0.0)), std::sqrt(std::fmax(xi[5 * 9 + 5], 0.0)),
+                          std::sqrt(std::fmax(xi[6 * 9 + 6], 0.0))};
+    pair_coef(rho0, cs2 - 1.0 / 3.0, kappa, -1.0 / tau_b, -1.0 / tau_s, -1.0 / tau_ghost, -1.0 / tau_ghost, L, s3, c,
+              rec);
     double co[6];
     noise_coefficients(rho0, cs2, kT, kappa, tau_s, tau_b, tau_ghost, co);
     rec->a44 = (float)co[0]; rec->b44 = (float)co[1];
@@ -436,14 +458,16 @@ void fill_rep_record(double rho0, double cs2, double kT, double kappa, double ta
     rec->a99 = (float)co[4]; rec->b99 = (float)co[5];
     // real-space correlated noise: Cholesky factors of the (4,9) block at k^2 = 0, 4, 16/3, / 4
     const double sk[3] = {0.0, 4.0, 16.0 / 3.0};
+    double sL[3][4];
     for (int j = 0; j < 3; ++j) {
         const double y44 = co[0] + co[1] * sk[j], y49 = co[2] + co[3] * sk[j], y99 = co[4] + co[5] * sk[j];
         const double l11 = std::sqrt(std::fmax(y44, 0.0));
         const double l21 = l11 > 0.0 ? y49 / l11 : 0.0;
         const double l22 = std::sqrt(std::fmax(y99 - l21 * l21, 0.0));
-        rec->sL[j][0] = (float)(0.25 * l11); rec->sL[j][1] = 0.0f;
-        rec->sL[j][2] = (float)(0.25 * l21); rec->sL[j][3] = (float)(0.25 * l22);
+        sL[j][0] = 0.25 * l11; sL[j][1] = 0.0;
+        sL[j][2] = 0.25 * l21; sL[j][3] = 0.25 * l22;
     }
+    pair_stencil(sL, c, rec);
     rec->mode = (noise_mode == LB_NOISE_OFF || kT <= 0.0)
                     ? 0
                     : (noise_mode == LB_NOISE_FULL ? 2 : (noise_mode == LB_NOISE_FULL_RS ? 3 : 1));
@@ -614,7 +638,7 @@ static int build_launches(lb_batch* b, int tile, std::vector<EnsParams>* out) {
         for (int j = 0; j < MAX_CLASSES && c0 + j < nc; ++j) {
             const ClassInfo& ci = b->L.classes[c0 + j];
             for (int w = 0; w < 2; ++w)
-                if (!make_class_map(cls_ptr(b, ci.off_buf[w]), ci.g, ci.R, tile, &p.map[j][w]))
+                if (!make_class_maps(cls_ptr(b, ci.off_buf[w]), ci.g, ci.R, tile, &p.map[j][w], &p.out[j][w]))
                     return bfail(b, LB_ECUDA, "cuTensorMapEncodeTiled failed for a size class");
             ClassDesc& d = p.cls[j];
             d.g = ci.g;
@@ -783,9 +807,6 @@ int lb_batch_create(int count, const int* nx, const int* ny, const uint64_t* see
     b->have_params.assign(count, false);
     for (int r = 0; r < count; ++r) {
         RepRec& rc = b->recs[r];
-        rc.rho0 = (float)rho0;
-        rc.cs2m = (float)(cs2 - SIGMA_S2_B);
-        rc.lb = rc.ls = rc.lq = rc.le = -1.0f;
         rc.k0 = (uint32_t)(seeds[r] & 0xffffffffu);
         rc.k1 = (uint32_t)(seeds[r] >> 32);
     }

@@ -42,20 +42,29 @@ struct SlotDesc {
 };
 
 struct ServeParams {
-    const CUtensorMap* maps;     // [slot][2], maps of buffers 0 and 1
+    const CUtensorMap* maps;     // [slot][4]: load maps of buffers 0 and 1, then their store maps
     const SlotDesc* desc;
     const RepRec* recs;
     const int* active;           // slots of this chunk
     const int* tile_begin;       // first tile of each active slot, ntiles at the end
+    int4* tiles;                 // [ntiles]: slot, x0, y0 of each tile (serve_tiles_kernel)
     int nactive, ntiles;
     long long* kstep;            // server step counter K (device)
     unsigned int* done;
     int* err;
 };
 
-// tile of the served kernel: 64 x 16 nodes on 512 threads (measured against 64 x 8 on 256:
-// faster on the request stream and on a large lattice alone, slower on a lone 256^2 one)
-constexpr int SV_TX = 64, SV_TY = 16, SV_NT = 512;
+// tile of the served kernel: 32 x 16 nodes on 128 threads, two rows of pairs a thread, the record's
+// coefficients read once for both (eight lattices of 1024^2: 153 us a step with scalar nodes on 64 x 16
+// tiles and 512 threads, 140 with this form; 3 x 512^2 20.8 and 18.7)
+constexpr int SV_TX = 32, SV_TY = 16, SV_NT = 128;
+constexpr int SV_GX = 32;            // ghost columns per side of every served lattice
+
+// its dynamic shared memory
+template <bool RS>
+constexpr int serve_smem() {
+    return TmaTile<SV_TX, SV_TY, float>::SMEM_BYTES + (RS ? StencilTile<SV_TX, SV_TY, SV_NT>::BYTES : 0);
+}
 
 // index of the active slot that owns `tile`: the last a with tile_begin[a] <= tile
 __device__ __forceinline__ int find_owner(const int* __restrict__ tile_begin, int n, int tile) {
@@ -68,123 +77,144 @@ __device__ __forceinline__ int find_owner(const int* __restrict__ tile_begin, in
     return lo;
 }
 
+// The slot and origin of every tile of a chunk, once per chunk: a step reads one record per tile,
+// a turn ahead, where a binary search over the active slots and three dependent loads per tile sat
+// between a tile's density pass and the next tile's load (8 lattices of 1024^2: 199 us a step).
+__global__ void serve_tiles_kernel(const ServeParams p, int tx, int ty) {
+    const int tile = blockIdx.x * blockDim.x + threadIdx.x;
+    if (tile >= p.ntiles) return;
+    const int a = find_owner(p.tile_begin, p.nactive, tile);
+    const int slot = p.active[a], rel = tile - p.tile_begin[a], ntx = p.desc[slot].ntx;
+    const int row = rel / ntx;
+    p.tiles[tile] = make_int4(slot, (rel - row * ntx) * tx, row * ty, 0);
+}
+
 // RS: the variant that also steps simulations with real-space correlated noise (launched
 // for chunks that hold one; its extra path raises the register count)
 template <int TX, int TY, int NT, bool RS>
-__global__ void __launch_bounds__(NT, 1024 / NT) step_serve_kernel(const ServeParams p) {
+__global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_serve_kernel(const ServeParams p) {
     using TT = TmaTile<TX, TY, float>;
+    using M = PairMap<TX, TY, NT>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    float* smem = reinterpret_cast<float*>(smem_raw);
-    float* R = reinterpret_cast<float*>(smem_raw + 2 * TT::STAGE_BYTES);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(R + TT::RW * TT::RH);
-    __shared__ int st_slot[2], st_x0[2], st_y0[2];
+    float* S = reinterpret_cast<float*>(smem_raw);
+    float* out = reinterpret_cast<float*>(smem_raw + TT::OUT);
+    float* R = reinterpret_cast<float*>(smem_raw + TT::RHO);
+    const uint32_t bar = smem_u32(smem_raw + TT::BAR);
+    unsigned char* xch = smem_raw + TT::SMEM_BYTES;     // RS: StencilTile
+    __shared__ int st_slot[2], st_x0[2], st_y0[2];      // of the tiles of even and odd turns
     __shared__ TileArgsOf<RS> sargs;    // the record of the current tile
-    __shared__ int smode;
     const int tid = threadIdx.x;
-    const long long K = __ldcg(p.kstep);
     const int ntiles = p.ntiles;
 
     if (tid == 0) {
-        mbar_init(smem_u32(&mbar[0]), 1);
-        mbar_init(smem_u32(&mbar[1]), 1);
+        mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    const long long K = __ldcg(p.kstep);
 
-    // thread 0: resolve the tile's slot and origin, remember them for the stage, load it
-    auto issue = [&](int tile, int s) {
-        const int a = find_owner(p.tile_begin, p.nactive, tile);
-        const int slot = __ldg(&p.active[a]);
-        const int rel = tile - __ldg(&p.tile_begin[a]);
-        const SlotDesc* d = p.desc + slot;
-        const int ntx = __ldg(&d->ntx);
-        const int ty = rel / ntx;
-        const int x0 = (rel - ty * ntx) * TX, y0 = ty * TY;
-        const long long sl = K - __ldg(&d->k_start);
-        const CUtensorMap* map = p.maps + 2 * slot + (int)(sl & 1);
-        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
-        st_slot[s] = slot;
-        st_x0[s] = x0;
-        st_y0[s] = y0;
-        const int gx = __ldg(&d->g.gx);
-        const uint32_t bar = smem_u32(&mbar[s]);
+    // thread 0: the record of a tile, and its slot's maps for this step, their descriptors made
+    // visible when the slot changes (the host writes them between launches)
+    int4 next = make_int4(-1, 0, 0, 0);
+    int seen = -1;
+    const CUtensorMap *lmap = nullptr, *smap = nullptr, *smap_next = nullptr;
+    auto resolve = [&](int tile) {
+        next = __ldg(&p.tiles[tile]);
+        const long long sl = K - __ldg(&p.desc[next.x].k_start);
+        lmap = p.maps + 4 * next.x + (int)(sl & 1);
+        smap_next = p.maps + 4 * next.x + 2 + (int)((sl & 1) ^ 1);
+        if (next.x != seen) {
+            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(lmap) : "memory");
+            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(smap_next) : "memory");
+            seen = next.x;
+        }
+    };
+    // thread 0: load the resolved tile for turn s
+    auto load = [&](int s) {
+        st_slot[s] = next.x;
+        st_x0[s] = next.y;
+        st_y0[s] = next.z;
         mbar_expect_tx(bar, TT::TX_BYTES);
-        float* st = smem + s * TT::STAGE;
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            tma_load_3d(smem_u32(st + i * TT::PS), map, x0 - TT::XO + gx, y0 - 1 - kCYt[i] + GY, i, bar);
+            tma_load_3d(smem_u32(S + i * TT::PS), lmap, next.y - TT::XO + SV_GX, next.z - 1 - kCYt[i] + GY, i, bar);
+    };
+    // thread 0: the results of the tile of turn s leave (smap: its slot's store map)
+    auto store = [&](int s) {
+        Grid g;
+        g.nx = __ldg(&p.desc[st_slot[s]].g.nx);
+        if (tile_direct<TX, float>(g, st_x0[s])) return;
+        tma_store_3d(smap, smem_u32(out), st_x0[s], st_y0[s], 0);
+        tma_store_commit();
     };
 
     const int first = blockIdx.x;
-    if (tid == 0) {
-        if (first < ntiles) issue(first, 0);
-        if (first + (int)gridDim.x < ntiles) issue(first + gridDim.x, 1);
+    if (tid == 0 && first < ntiles) {
+        resolve(first);
+        load(0);
     }
-    __syncthreads();   // the slots and origins of the first two tiles are visible to all
-    int k = 0;
+    uint32_t k = 0;
     for (int tile = first; tile < ntiles; tile += gridDim.x, ++k) {
-        const int s = k & 1;
-        // the tile's slot and origin (written before the previous barrier) are read while
-        // its populations are in flight
-        const int slot = st_slot[s], x0 = st_x0[s], y0 = st_y0[s];
-        const SlotDesc* d = p.desc + slot;
-        const long long sl = K - __ldg(&d->k_start);
-        const bool ok = mbar_wait_bounded(smem_u32(&mbar[s]), (uint32_t)((k >> 1) & 1));
+        const int s = (int)(k & 1u);
+        const CUtensorMap* smap_cur = smap_next;       // of this tile
+        if (tid == 0 && tile + (int)gridDim.x < ntiles) resolve(tile + gridDim.x);
+        const bool ok = mbar_wait_bounded(bar, k & 1u);
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 atomicExch(p.err, 1);
-                mbar_wait_bounded(smem_u32(&mbar[s]), (uint32_t)((k >> 1) & 1));
-                if (tile + (int)gridDim.x < ntiles)
-                    mbar_wait_bounded(smem_u32(&mbar[s ^ 1]), (uint32_t)(((k + 1) >> 1) & 1));
+                mbar_wait_bounded(bar, k & 1u);
             }
+            k = 0;                     // nothing of this CTA is left to store
             break;
         }
+        if (tid == 0 && k > 0) store(s ^ 1);
+        smap = smap_cur;
+        // the tile's slot and origin (written before the barrier above)
+        const int slot = st_slot[s], x0 = st_x0[s], y0 = st_y0[s];
+        const SlotDesc* d = p.desc + slot;
+        const long long sl = K - __ldg(&d->k_start);
         Grid g;
         g.nx = __ldg(&d->g.nx); g.ny = __ldg(&d->g.ny); g.gx = __ldg(&d->g.gx);
         g.pitch = __ldg(&d->g.pitch); g.plane = __ldg(&d->g.plane);
         float* dst = (sl & 1) ? d->buf[0] : d->buf[1];
-        const float* S = smem + s * TT::STAGE;
         // the slot's record, to shared memory (its last readers, the previous tile's
         // collision, are past the barrier above)
-        if (tid == 0) {
-            load_tile_args(p.recs + slot, sl, &sargs, &smode);
-            if constexpr (RS) {
-                if (smode == 3) load_stencil_args(p.recs + slot, &sargs);
-            }
-        }
+        load_tile_args<RS>(p.recs + slot, sl, &sargs);
 
-        // pulled populations stay in registers across the density barrier; the stage is
-        // refilled right after it (slot, x0, y0 are in registers by then)
-        float fr[TX * TY / NT][Q];
-        tile_pull<TX, TY, NT, RS>(S, R, fr);
+        // pulled populations stay in registers across the density barrier; the next tile is
+        // loaded right after it (the other turn's slot and origin, read by the store above, are free)
+        F2 fr[M::RPT][Q], z4[M::RPT], z9[M::RPT];
+        tile_pull<TX, TY, NT, false, RS>(S, R, fr);
+        if (tid == 0) tma_store_wait_read();
         __syncthreads();
-        const int mode = smode;
-        if (tid == 0 && !(RS && mode == 3) && tile + 2 * (int)gridDim.x < ntiles) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue(tile + 2 * gridDim.x, s);
+        const int mode = sargs.mode;        // the tile's: uniform over the CTA
+        if (tid == 0 && tile + (int)gridDim.x < ntiles) {
+            fence_async_smem();
+            load(s ^ 1);
         }
         bool stepped = false;
         if constexpr (RS) {
             if (mode == 3) {
-                // real-space correlated noise: contributions in the consumed stage s, refilled
-                // after the collision (the mode is the tile's: uniform over the CTA)
-                float2* Hs = reinterpret_cast<float2*>(smem_raw + s * TT::STAGE_BYTES);
-                tile_stencil<TX, TY, NT>(sargs, Hs, g, x0, y0);
+                stencil_tile<TX, TY, NT>(sargs, xch, x0, y0, g.nx, g.ny, z4, z9);
                 __syncthreads();
-                tile_nodes<3, TX, TY, NT>(sargs, fr, R, g, x0, y0, dst, nullptr, Hs);
-                __syncthreads();
-                if (tid == 0 && tile + 2 * (int)gridDim.x < ntiles) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    issue(tile + 2 * gridDim.x, s);
-                }
+                tile_collide<3, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, xch);
                 stepped = true;
             }
         }
         if (!stepped) {
-            if (mode == 2) tile_nodes<2, TX, TY, NT>(sargs, fr, R, g, x0, y0, dst, d->xi);
-            else if (mode) tile_nodes<1, TX, TY, NT>(sargs, fr, R, g, x0, y0, dst, nullptr);
-            else tile_nodes<0, TX, TY, NT>(sargs, fr, R, g, x0, y0, dst, nullptr);
+            if (mode == 2)
+                tile_collide<2, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, d->xi, z4, z9, nullptr);
+            else if (mode)
+                tile_collide<1, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, nullptr);
+            else
+                tile_collide<0, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, nullptr);
         }
+        fence_async_smem();
+    }
+    __syncthreads();
+    if (tid == 0 && k > 0) {
+        store((int)((k - 1u) & 1u));
+        tma_store_wait();
     }
     if (tid == 0) {
         const unsigned int prev = atomicAdd(p.done, 1u);
@@ -241,17 +271,25 @@ __global__ void __launch_bounds__(1024) serve_noise_rows_kernel(const int* __res
     }
 }
 
-static bool make_slot_map(void* buf, const Grid& g, CUtensorMap* map) {
+// load and store maps of one population buffer of a slot (make_pop_tensor_maps of
+// lb_step_tma.cu for the served tile)
+static bool make_slot_maps(void* buf, const Grid& g, CUtensorMap* load, CUtensorMap* store) {
     EncodeTiledFn fn = tensor_map_encoder();
     if (!fn) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)g.pitch, (cuuint64_t)(g.ny + 2 * GY), (cuuint64_t)Q};
     cuuint64_t strides[2] = {(cuuint64_t)g.pitch * 4, (cuuint64_t)g.plane * 4};
-    cuuint32_t box[3] = {(cuuint32_t)(SV_TX + 8), (cuuint32_t)(SV_TY + 2), 1};
     cuuint32_t estr[3] = {1, 1, 1};
+    cuuint64_t ldims[3] = {(cuuint64_t)g.pitch, (cuuint64_t)(g.ny + 2 * GY), (cuuint64_t)Q};
+    cuuint32_t lbox[3] = {(cuuint32_t)(SV_TX + 8), (cuuint32_t)(SV_TY + 2), 1};
     // 64-byte L2 promotion, as for the batched engine's class maps (lb_batch.cu): the slot's
     // ghost columns are mostly never read
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, buf, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_64B,
+    if (fn(load, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, buf, ldims, strides, lbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+           CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_64B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
+        CUDA_SUCCESS)
+        return false;
+    cuuint64_t sdims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)Q};
+    cuuint32_t sbox[3] = {(cuuint32_t)SV_TX, (cuuint32_t)SV_TY, (cuuint32_t)Q};
+    return fn(store, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (float*)buf + g.at(0, 0), sdims, strides, sbox, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -261,15 +299,13 @@ using namespace lbf;
 
 namespace {
 
-constexpr double SIGMA_S2_S = 1.0 / 3.0;
-
 using Clock = std::chrono::steady_clock;
 
 size_t align256s(size_t v) { return (v + 255) & ~size_t(255); }
 
 bool serve_grid(int nx, int ny, Grid* g) {
     if (nx < 2 || ny < 2 || nx > 16384 || ny > 16384) return false;
-    g->nx = nx; g->ny = ny; g->gx = 32;
+    g->nx = nx; g->ny = ny; g->gx = SV_GX;
     g->pitch = (nx + 64 + 31) / 32 * 32;
     g->plane = ((long long)g->pitch * (ny + 2 * GY) + 63) / 64 * 64;
     return true;
@@ -343,6 +379,8 @@ struct lb_server {
     std::map<std::pair<int, int>, SizeTables> tables;
     size_t noise_csm = 0, noise_rsm = 0;     // shared memory the noise kernels are set up for
     int* d_tb[2] = {nullptr, nullptr};
+    int4* d_tiles = nullptr;                 // tile records of the current chunk (grown on demand)
+    int tiles_cap = 0;
     long long* d_k = nullptr;
     unsigned int* d_done = nullptr;
     int* d_err = nullptr;
@@ -352,7 +390,7 @@ struct lb_server {
     int* h_tb[2] = {nullptr, nullptr};
     double* h_sums = nullptr;        // [slot][3]
     int* h_err = nullptr;            // [2]: error word after the chunk of that parity
-    unsigned char* h_slot = nullptr; // per slot: 2 maps, desc, record, fbar
+    unsigned char* h_slot = nullptr; // per slot: 4 maps, desc, record, fbar
     size_t slot_stage = 0;
     // scheduling state (worker thread)
     std::vector<int> free_slots;
@@ -578,12 +616,12 @@ bool admit(lb_server* s) {
         float* b1 = reinterpret_cast<float*>(run.mem + buf_bytes(run.g));
         unsigned char* st = slot_stage(s, run.slot);
         CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(st);
-        if (!make_slot_map(b0, run.g, &maps[0]) || !make_slot_map(b1, run.g, &maps[1])) {
+        if (!make_slot_maps(b0, run.g, &maps[0], &maps[2]) || !make_slot_maps(b1, run.g, &maps[1], &maps[3])) {
             std::lock_guard<std::mutex> lk(s->mu);
             s->err = "cuTensorMapEncodeTiled failed";
             return false;
         }
-        SlotDesc* d = reinterpret_cast<SlotDesc*>(st + 2 * sizeof(CUtensorMap));
+        SlotDesc* d = reinterpret_cast<SlotDesc*>(st + 4 * sizeof(CUtensorMap));
         d->g = run.g;
         d->buf[0] = b0;
         d->buf[1] = b1;
@@ -594,18 +632,16 @@ bool admit(lb_server* s) {
         }
         d->ntx = (run.g.nx + SV_TX - 1) / SV_TX;
         d->k_start = s->K;
-        RepRec* rec = reinterpret_cast<RepRec*>(st + 2 * sizeof(CUtensorMap) + sizeof(SlotDesc));
+        RepRec* rec = reinterpret_cast<RepRec*>(st + 4 * sizeof(CUtensorMap) + sizeof(SlotDesc));
         std::memset(rec, 0, sizeof(RepRec));
-        rec->rho0 = (float)pr.r.rho0;
-        rec->cs2m = (float)(pr.r.cs2 - SIGMA_S2_S);
         fill_rep_record(pr.r.rho0, pr.r.cs2, pr.r.kT, pr.r.kappa, pr.r.tau_s, pr.r.tau_b, pr.r.tau_ghost,
                         pr.r.noise_mode, rec);
         rec->k0 = (uint32_t)(pr.r.seed & 0xffffffffu);
         rec->k1 = (uint32_t)(pr.r.seed >> 32);
         rec->toff = 0;
-        double* fb = reinterpret_cast<double*>(st + 2 * sizeof(CUtensorMap) + sizeof(SlotDesc) + sizeof(RepRec));
+        double* fb = reinterpret_cast<double*>(st + 4 * sizeof(CUtensorMap) + sizeof(SlotDesc) + sizeof(RepRec));
         rest_populations(pr.r.rho0, pr.r.cs2, fb);
-        SCK(s, cudaMemcpyAsync(s->d_maps + 2 * run.slot, maps, 2 * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
+        SCK(s, cudaMemcpyAsync(s->d_maps + 4 * run.slot, maps, 4 * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
                                s->stream));
         SCK(s, cudaMemcpyAsync(s->d_desc + run.slot, d, sizeof(SlotDesc), cudaMemcpyHostToDevice, s->stream));
         SCK(s, cudaMemcpyAsync(s->d_recs + run.slot, rec, sizeof(RepRec), cudaMemcpyHostToDevice, s->stream));
@@ -719,7 +755,17 @@ bool issue_chunk(lb_server* s) {
     p.kstep = s->d_k;
     p.done = s->d_done;
     p.err = s->d_err;
-    using TT = TmaTile<SV_TX, SV_TY, float>;
+    if (tiles > s->tiles_cap) {
+        // 16 bytes per 512 nodes; earlier chunks' launches are ahead in the stream
+        if (s->d_tiles) SCK(s, cudaFreeAsync(s->d_tiles, s->stream));
+        s->d_tiles = nullptr;
+        s->tiles_cap = 0;
+        const int cap = std::max(4096, tiles + tiles / 2);
+        SCK(s, cudaMallocFromPoolAsync((void**)&s->d_tiles, (size_t)cap * sizeof(int4), s->pool, s->stream));
+        s->tiles_cap = cap;
+    }
+    p.tiles = s->d_tiles;
+    serve_tiles_kernel<<<(tiles + 255) / 256, 256, 0, s->stream>>>(p, SV_TX, SV_TY);
     bool rs = false;
     for (const Running& r : s->running) rs = rs || (r.r.noise_mode == LB_NOISE_FULL_RS && r.r.kT > 0.0);
     const int grid = std::max(1, std::min(tiles, rs ? s->grid_rs : s->grid));
@@ -735,8 +781,8 @@ bool issue_chunk(lb_server* s) {
                 s->d_full[c] + gr.off, s->d_desc, gr.nx, gr.ny, tb2.twx,
                 (float)(1.0 / std::sqrt((double)gr.nx * gr.ny)));
         }
-        if (rs) step_serve_kernel<SV_TX, SV_TY, SV_NT, true><<<grid, SV_NT, TT::SMEM_BYTES, s->stream>>>(p);
-        else step_serve_kernel<SV_TX, SV_TY, SV_NT, false><<<grid, SV_NT, TT::SMEM_BYTES, s->stream>>>(p);
+        if (rs) step_serve_kernel<SV_TX, SV_TY, SV_NT, true><<<grid, SV_NT, serve_smem<true>(), s->stream>>>(p);
+        else step_serve_kernel<SV_TX, SV_TY, SV_NT, false><<<grid, SV_NT, serve_smem<false>(), s->stream>>>(p);
     }
     SCK(s, cudaGetLastError());
     s->K += G;
@@ -833,7 +879,7 @@ int lb_server_create(size_t hbm_budget_bytes, int max_active, int max_chunk_step
     s->max_chunk = max_chunk_steps;
     s->t0 = Clock::now();
     cudaGetDevice(&s->device);
-    s->slot_stage = align256s(2 * sizeof(CUtensorMap) + sizeof(SlotDesc) + sizeof(RepRec) + Q * sizeof(double));
+    s->slot_stage = align256s(4 * sizeof(CUtensorMap) + sizeof(SlotDesc) + sizeof(RepRec) + Q * sizeof(double));
     auto fail_create = [&](cudaError_t e) {
         set_context_free_error(std::string("lb_server_create: ") + cudaGetErrorString(e));
         lb_server_destroy(s);
@@ -851,7 +897,7 @@ int lb_server_create(size_t hbm_budget_bytes, int max_active, int max_chunk_step
     if ((e = cudaMemPoolSetAttribute(s->pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess)
         return fail_create(e);
     const size_t M = (size_t)max_active;
-    if ((e = cudaMalloc(&s->d_maps, M * 2 * sizeof(CUtensorMap))) != cudaSuccess) return fail_create(e);
+    if ((e = cudaMalloc(&s->d_maps, M * 4 * sizeof(CUtensorMap))) != cudaSuccess) return fail_create(e);
     if ((e = cudaMalloc(&s->d_desc, M * sizeof(SlotDesc))) != cudaSuccess) return fail_create(e);
     if ((e = cudaMalloc(&s->d_recs, M * sizeof(RepRec))) != cudaSuccess) return fail_create(e);
     if ((e = cudaMalloc(&s->d_fbar, M * Q * sizeof(double))) != cudaSuccess) return fail_create(e);
@@ -881,16 +927,16 @@ int lb_server_create(size_t hbm_budget_bytes, int max_active, int max_chunk_step
     using TT = TmaTile<SV_TX, SV_TY, float>;
     auto kern = step_serve_kernel<SV_TX, SV_TY, SV_NT, false>;
     auto kern_rs = step_serve_kernel<SV_TX, SV_TY, SV_NT, true>;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TT::SMEM_BYTES)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, serve_smem<false>())) != cudaSuccess)
         return fail_create(e);
-    if ((e = cudaFuncSetAttribute(kern_rs, cudaFuncAttributeMaxDynamicSharedMemorySize, TT::SMEM_BYTES)) !=
+    if ((e = cudaFuncSetAttribute(kern_rs, cudaFuncAttributeMaxDynamicSharedMemorySize, serve_smem<true>())) !=
         cudaSuccess)
         return fail_create(e);
     int sms = 0, per = 0, per_rs = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, SV_NT, TT::SMEM_BYTES)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, SV_NT, serve_smem<false>())) != cudaSuccess)
         return fail_create(e);
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_rs, kern_rs, SV_NT, TT::SMEM_BYTES)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_rs, kern_rs, SV_NT, serve_smem<true>())) != cudaSuccess)
         return fail_create(e);
     s->grid = sms * std::max(per, 1);
     s->grid_rs = sms * std::max(per_rs, 1);
@@ -1081,6 +1127,7 @@ int lb_server_destroy(lb_server* s) {
     if (s->stream) cudaStreamSynchronize(s->stream);
     for (auto& kv : s->kept) cudaFreeAsync(kv.second.run.mem, s->stream);
     for (auto& r : s->running) cudaFreeAsync(r.mem, s->stream);
+    if (s->d_tiles) cudaFreeAsync(s->d_tiles, s->stream);
     if (s->stream) cudaStreamSynchronize(s->stream);
     cudaFree(s->d_maps); cudaFree(s->d_desc); cudaFree(s->d_recs); cudaFree(s->d_fbar); cudaFree(s->d_sums);
     for (int c = 0; c < 2; ++c) {

@@ -1,6 +1,7 @@
 // lb_step_tma.cu -- the fused fluctuating D2Q9 step, TMA-staged and persistent.
 //
-// Same arithmetic as lb_step.cu (collide_node), different data movement:
+// Same arithmetic as lb_step.cu (collide_node), two nodes at a time (collide_pair of lb_pair.cuh),
+// and different data movement:
 //   * a persistent grid (resident CTAs only) walks the lattice in TX x TY tiles (the shape
 //     chosen per noise mode and storage, tma_default_tile) in row-major tile order, so the
 //     tiles in flight form a band whose halo rows are still in L2 when the neighbouring tile
@@ -10,184 +11,143 @@
 //     into shared memory; the y offset of plane i absorbs its streaming shift, so node
 //     (lx, ly) of the tile reads f_i at box[ly + 1][lx + 4 - cx_i].  The x start is rounded
 //     down to a 16-byte boundary (four floats) as TMA requires;
-//   * two stages and an mbarrier each: tile k+1 is in flight while tile k is computed;
-//   * every thread pulls its nodes' nine deviations from shared memory into registers and
+//   * every thread pulls its pairs' nine deviations from shared memory into registers and
 //     writes their density to a tile-plus-ring array (the ring from the halo); after one
-//     barrier the stage is refilled with the tile two steps ahead while every node
-//     collides and stores its nine post-collision deviations (and periodic ghosts)
-//     directly from registers with coalesced stores.  Nodes beyond a ragged edge of the
-//     lattice take part in the density pass (their values are never used) but not in the
-//     collision pass.
+//     barrier the next tile is loaded into the same stage while every pair collides.  Nodes
+//     beyond a ragged edge of the lattice take part in the density pass (their values are
+//     never used);
+//   * the post-collision planes go to a tile in shared memory, which leaves with one TMA store
+//     (a box of nine planes, clipped to the lattice) behind the next tile's density pass; the
+//     periodic ghost copies of a tile near an edge are stored by its threads.
+//
+// One load in flight per CTA, not two: with the tile after next requested early the 4096^2 step
+// had 190 KB of requests outstanding per SM, and DRAM then answers more slowly (no noise 250 us
+// against 191 on the same tiles; a plain copy of nine planes shows the same, 183 us with 55 KB
+// in flight per SM and 233 us with 147 KB).
+//
+// Step at 4096^2, before and after this form (scalar nodes, two stages, stores by thread):
+// FP32 without noise 262 -> 186 us, uncorrelated 212 -> 191 (6.32 TB/s of the 72 bytes a node),
+// k-space correlated (the step kernel) 235 -> 221 less launch, real space 333 -> 263, local
+// density 219 -> 194; FP16 uncorrelated 220 -> 182, 209 instructions a node against 341.  What
+// bounds it now: FP32 DRAM; FP16 and the real-space noise the SM (FMA-heavy pipe 60 % busy, half
+// of it the wide multiplies of Philox, and the barriers between the passes).
+//
 // Waits on the mbarriers are bounded by the global timer; a CTA that gives up sets the
 // error word, gives its loads in flight a bounded chance to land, and returns.
 #include <cuda.h>
 
 #include <type_traits>
 
-#include "lb_collide.cuh"
-#include "lb_tma.cuh"
+#include "lb_pair.cuh"
 
 namespace lbf {
 
-struct TmaArgs {
-    StepArgs a;
+// What one launch reads, by value: the lattice's coefficients as lb_pair.cuh takes them, the
+// time and the Philox round keys.
+struct TmaArgs : PairCoef, PairStencil {
+    PairLocal loc;     // POLY and MODE 4
+    Grid g;
+    void* dst;
+    const float2* xi49;
     int ntx, nty;      // tiles along x and y
     int* err;          // device error word (1 = a TMA wait timed out)
+    uint32_t t_lo, t_hi;
+    RoundKeys rk;
 };
 
-
-// POLY: the double-well equation of state (the bulk pressure's quartic in drho, StepArgs e2..e4)
+// POLY: the double-well equation of state (the bulk pressure's quartic in drho)
 template <int TX, int TY, int NT, int MODE, typename T, bool POLY = false>
-__global__ void __launch_bounds__(NT) step_tma_kernel(const __grid_constant__ CUtensorMap tmap, const TmaArgs ta) {
+__global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>()))
+    step_tma_kernel(const __grid_constant__ CUtensorMap lmap, const __grid_constant__ CUtensorMap smap,
+                    const TmaArgs a) {
     using TT = TmaTile<TX, TY, T>;
+    using M = PairMap<TX, TY, NT>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    T* smem = reinterpret_cast<T*>(smem_raw);
-    float* R = reinterpret_cast<float*>(smem_raw + 2 * TT::STAGE_BYTES);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(R + TT::RW * TT::RH);
-    const StepArgs& a = ta.a;
+    T* S = reinterpret_cast<T*>(smem_raw);
+    T* out = reinterpret_cast<T*>(smem_raw + TT::OUT);
+    float* R = reinterpret_cast<float*>(smem_raw + TT::RHO);
+    const uint32_t bar = smem_u32(smem_raw + TT::BAR);
+    unsigned char* xch = smem_raw + TT::SMEM_BYTES;     // MODE 3: StencilTile
     const Grid g = a.g;
     const int tid = threadIdx.x;
-    const int ntiles = ta.ntx * ta.nty;
+    const int ntiles = a.ntx * a.nty;
     // FP16 storage collides in the stored form g_i = df_i / w_i (no scaling on load or store)
     constexpr bool GF = std::is_same<T, __half>::value;
-    auto load9 = [](const T* S, int b, float f[Q]) { load9_ps<TT::PS, T, GF>(S, b, f); };
-    auto rho_of = [](const float f[Q]) { return GF ? drho_of_g(f) : drho_of(f); };
-    // MODE 3: the 2 x 2-box noise contributions, after the mbarriers (kept apart from the
-    // stages: filling them into the consumed stage and refilling it after the collision
-    // measured slower, the two extra barriers costing more than the fourth CTA per SM gained)
-    float2* H = reinterpret_cast<float2*>(smem_raw + TT::H_OFFSET);
 
     if (tid == 0) {
-        mbar_init(smem_u32(&mbar[0]), 1);
-        mbar_init(smem_u32(&mbar[1]), 1);
+        mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&lmap)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&smap)) : "memory");
     }
     __syncthreads();
 
-    // the nine boxes of the tile in column col, row row of the tiling into stage s
-    auto issue = [&](int col, int row, int s) {
+    // the nine boxes of the tile in column col, row row of the tiling
+    auto load = [&](int col, int row) {
         const int x0 = col * TX, y0 = row * TY;
-        const uint32_t bar = smem_u32(&mbar[s]);
         mbar_expect_tx(bar, TT::TX_BYTES);
-        T* st = smem + s * TT::STAGE;
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            tma_load_3d(smem_u32(st + i * TT::PS), &tmap, x0 - TT::XO + g.gx, y0 - 1 - kCYt[i] + GY, i, bar);
+            tma_load_3d(smem_u32(S + i * TT::PS), &lmap, x0 - TT::XO + g.gx, y0 - 1 - kCYt[i] + GY, i, bar);
     };
 
     // a tile's column and row, advanced by the grid stride without a division per tile
     const int first = blockIdx.x;
-    const int stx = (int)gridDim.x % ta.ntx, sty = (int)gridDim.x / ta.ntx;
-    auto advance = [&](int& col, int& row) {
-        col += stx;
-        row += sty;
-        if (col >= ta.ntx) {
-            col -= ta.ntx;
-            ++row;
-        }
-    };
-    int tcol = first % ta.ntx, trow = first / ta.ntx;
-    if (tid == 0) {
-        if (first < ntiles) issue(tcol, trow, 0);
-        int c1 = tcol, r1 = trow;
-        advance(c1, r1);
-        if (first + (int)gridDim.x < ntiles) issue(c1, r1, 1);
-    }
-    int k = 0;
+    const int stx = (int)gridDim.x % a.ntx, sty = (int)gridDim.x / a.ntx;
+    int tcol = first % a.ntx, trow = first / a.ntx;
+    if (tid == 0 && first < ntiles) load(tcol, trow);
+    int px0 = 0, py0 = 0;                  // the tile whose results are in `out`
+    uint32_t k = 0;
     for (int tile = first; tile < ntiles; tile += gridDim.x, ++k) {
-        const int s = k & 1;
-        const uint32_t parity = (uint32_t)((k >> 1) & 1);
-        // bounded wait for this tile's nine boxes; the decision to give up is collective
-        // (this barrier also orders the previous tile's reads of R before this tile's writes)
-        const bool ok = mbar_wait_bounded(smem_u32(&mbar[s]), parity);
+        // bounded wait for this tile's nine boxes; the decision to give up is collective (the
+        // barrier also orders the previous tile's reads of R and writes of `out` before this
+        // tile's writes and the store)
+        const bool ok = mbar_wait_bounded(bar, k & 1u);
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
-                atomicExch(ta.err, 1);
+                atomicExch(a.err, 1);
                 // give the loads still in flight into this CTA's shared memory a bounded
                 // chance to land before the CTA exits
-                mbar_wait_bounded(smem_u32(&mbar[s]), parity);
-                if (tile + (int)gridDim.x < ntiles)
-                    mbar_wait_bounded(smem_u32(&mbar[s ^ 1]), (uint32_t)(((k + 1) >> 1) & 1));
+                mbar_wait_bounded(bar, k & 1u);
             }
             return;
         }
-        const T* S = smem + s * TT::STAGE;
+        if (tid == 0 && k > 0 && !tile_direct<TX, T>(g, px0)) {
+            tma_store_3d(&smap, smem_u32(out), px0, py0, 0);
+            tma_store_commit();
+        }
         const int x0 = tcol * TX, y0 = trow * TY;
-        advance(tcol, trow);        // now the next tile's
+        px0 = x0;
+        py0 = y0;
+        tcol += stx;                       // now the next tile's
+        trow += sty;
+        if (tcol >= a.ntx) {
+            tcol -= a.ntx;
+            ++trow;
+        }
 
-        static_assert((TX * TY) % NT == 0, "tile must be a multiple of the block");
-        constexpr int NN = TX * TY / NT;
-        // each thread pulls its nodes' nine deviations once, keeps them in registers across
-        // the barrier and writes their density to the tile; the ring is formed separately
-        float fr[NN][Q];
-#pragma unroll
-        for (int it = 0; it < NN; ++it) {
-            const int q = tid + it * NT;
-            const int ly = q / TX, lx = q - ly * TX;
-            load9(S, (ly + 1) * TT::BW + lx + TT::XO, fr[it]);
-            R[(ly + 1) * TT::RW + lx + 1] = rho_of(fr[it]);
-        }
-        // real-space correlated noise: every node's contributions, then the halo's
-        auto stencil_tile = [&](float2* Hd) {
-#pragma unroll 1
-            for (int it = 0; it < NN; ++it) {
-                const int q = tid + it * NT;
-                const int ly = q / TX, lx = q - ly * TX;
-                const int x = x0 + lx, y = y0 + ly;
-                if (x < g.nx && y < g.ny)
-                    stencil_store<TT::HW>(a, Hd, TT::HN, lx, ly, (uint32_t)y * (uint32_t)g.nx + (uint32_t)x);
-            }
-            stencil_halo<TX, TY, TT::HW>(a, Hd, TT::HN, x0, y0, g.nx, g.ny, tid, NT);
-        };
-        if (MODE == 3) stencil_tile(H);
-        // the ring: rows 0 and TY + 1 (TX + 2 each), then columns 0 and TX + 1, on the last
-        // threads (the first issues the refill); with MODE 3 on the first (the last form the
-        // noise contributions of the halo)
-        constexpr int NB = 2 * (TX + 2) + 2 * TY;
-        for (int j = MODE == 3 ? tid : NT - 1 - tid; j < NB; j += NT) {
-            int rx, ry;
-            if (j < TX + 2) { rx = j; ry = 0; }
-            else if (j < 2 * (TX + 2)) { rx = j - (TX + 2); ry = TY + 1; }
-            else { const int u = j - 2 * (TX + 2); ry = 1 + (u >> 1); rx = (u & 1) ? TX + 1 : 0; }
-            float h[Q];
-            load9(S, ry * TT::BW + rx + TT::XO - 1, h);
-            R[ry * TT::RW + rx] = rho_of(h);
-        }
+        // each thread pulls its pairs of nodes once, keeps them in registers across the barrier
+        // and writes their density to the tile; the ring is formed separately
+        F2 fr[M::RPT][Q];
+        tile_pull<TX, TY, NT, GF, MODE == 3>(S, R, fr);
+        F2 z4[M::RPT], z9[M::RPT];
+        if constexpr (MODE == 3) stencil_tile<TX, TY, NT>(a, xch, x0, y0, g.nx, g.ny, z4, z9);
+        if (tid == 0) tma_store_wait_read();
         __syncthreads();
-        // the collision pass reads no population from stage s: refill it now with the tile
-        // two steps ahead
-        if (tid == 0 && tile + 2 * (int)gridDim.x < ntiles) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            int c2 = tcol, r2 = trow;
-            advance(c2, r2);
-            issue(c2, r2, s);
+        // the collision pass reads no population from the stage: load the next tile now
+        if (tid == 0 && tile + (int)gridDim.x < ntiles) {
+            fence_async_smem();
+            load(tcol, trow);
         }
-
-        // collide every node of the tile; the nodes of one thread are independent, so
-        // their random-number and collision chains interleave
-#pragma unroll
-        for (int it = 0; it < NN; ++it) {
-            const int q = tid + it * NT;
-            const int ly = q / TX, lx = q - ly * TX;
-            const int x = x0 + lx, y = y0 + ly;
-            if (x >= g.nx || y >= g.ny) continue;
-            const float* f = fr[it];
-            const int rc = (ly + 1) * TT::RW + lx + 1;
-            Nbr r;
-            r.C = R[rc];
-            r.E = R[rc + 1]; r.W = R[rc - 1];
-            r.N = R[rc + TT::RW]; r.S = R[rc - TT::RW];
-            r.NE = R[rc + TT::RW + 1]; r.NW = R[rc + TT::RW - 1];
-            r.SE = R[rc - TT::RW + 1]; r.SW = R[rc - TT::RW - 1];
-            const uint32_t node = (uint32_t)y * (uint32_t)g.nx + (uint32_t)x;
-            float2 z = make_float2(0.f, 0.f);
-            if (MODE == 2) z = a.xi49[(long long)y * g.nx + x];
-            if (MODE == 3) z = stencil_xi<TT::HW>(H, TT::HN, lx, ly);
-            float o[Q];
-            collide_node<MODE, POLY, GF>(a, f, r, node, z, o);
-            store9<T, float, GF>(static_cast<T*>(a.dst), g.plane, g, x, y, o);
-        }
+        tile_collide<MODE, POLY, GF, TX, TY, NT>(a, &a.loc, fr, R, g, x0, y0, out, static_cast<T*>(a.dst), a.xi49, z4,
+                                                 z9, xch);
+        fence_async_smem();
+    }
+    __syncthreads();
+    if (tid == 0 && k > 0 && !tile_direct<TX, T>(g, px0)) {
+        tma_store_3d(&smap, smem_u32(out), px0, py0, 0);
+        tma_store_commit();
+        tma_store_wait();
     }
 }
 
@@ -210,57 +170,66 @@ static const int kTiles[5][3] = {{32, 16, 256}, {32, 32, 256}, {64, 8, 256}, {64
 
 int tma_tile_count() { return 5; }
 
-// The fastest shape per noise mode (0 off, 1 uncorrelated, 2 correlated, 3 correlated built
-// in real space) and storage, measured on GB300 at 4096^2: FP32 off 32x32 (263 us),
-// uncorrelated 32x32 (212.5 us against 214.1 for 64x16/512, alternating runs on one box),
-// correlated 32x16 (235.0 us; 32x32 285, 64x16 240), real space 32x16 (334 us; 32x32 422);
-// FP16 off 32x16/128 (153 us), uncorrelated 32x32 (220.1 us; the others 221-226),
-// correlated 64x16 (245 us).
+// The fastest shape per noise mode (0 off, 1 uncorrelated, 2 correlated, 3 correlated built in real
+// space, 4 local density) and storage, measured at 4096^2 (us a step, shapes 0 to 4):
+//   FP32 off 191 208 186 205 190, uncorrelated 194 213 191 209 193, correlated (kernel alone) 232 257
+//   221 225 229, real space 294 281 304 402 263, local 195 218 194 211 198;
+//   FP16 off 140 - 134 - 133, uncorrelated 186 185 183 188 182, real space 300 - 312 - 276.
+// Four CTAs per SM hide each other's barriers: one pair a thread where the registers allow 32 warps
+// (shape 2), two pairs and 16 warps where the contributions of the real-space noise need them
+// (shape 4: their exchange stays within a thread for half the rows).  2048^2 and 3000^2 agree; below
+// 512^2 a step is bound by its launch and the shape does not matter.
 int tma_default_tile(int noise_mode, int fp16) {
-    static const int best[2][5] = {{1, 1, 0, 0, 3}, {4, 1, 3, 0, 1}};
+    static const int best[2][5] = {{2, 2, 2, 4, 2}, {4, 4, 2, 4, 2}};
     const int m = noise_mode < 0 ? 0 : (noise_mode > 4 ? 4 : noise_mode);
     return best[fp16 ? 1 : 0][m];
 }
 
-// Tensor map over one population buffer: dims (pitch, ny + 2 GY, 9) of FP32, box
-// (TX + 8, TY + 2, 1), zero fill outside.
-bool make_pop_tensor_map(const void* buf, const Grid& g, int tile, int fp16, void* map_out) {
+// Tensor maps over one population buffer.  For loads: dims (pitch, ny + 2 GY, 9), a plane's box of
+// the tile with its halo.  For stores: dims (nx, ny, 9) from node (0, 0), so that a ragged tile is
+// clipped to the lattice, the nine planes of the tile in one box.
+bool make_pop_tensor_maps(const void* buf, const Grid& g, int tile, int fp16, void* load_map, void* store_map) {
     EncodeTiledFn fn = tensor_map_encoder();
     if (!fn || tile < 0 || tile >= tma_tile_count()) return false;
     const cuuint64_t es = fp16 ? 2 : 4;
     const int xo = fp16 ? Elem<__half>::XO : Elem<float>::XO;
-    cuuint64_t dims[3] = {(cuuint64_t)g.pitch, (cuuint64_t)(g.ny + 2 * GY), (cuuint64_t)Q};
+    const CUtensorMapDataType dt = fp16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     cuuint64_t strides[2] = {(cuuint64_t)g.pitch * es, (cuuint64_t)g.plane * es};
-    cuuint32_t box[3] = {(cuuint32_t)(kTiles[tile][0] + 2 * xo), (cuuint32_t)kTiles[tile][1] + 2, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(reinterpret_cast<CUtensorMap*>(map_out),
-                    fp16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)buf, dims,
-                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
+    cuuint64_t ldims[3] = {(cuuint64_t)g.pitch, (cuuint64_t)(g.ny + 2 * GY), (cuuint64_t)Q};
+    cuuint32_t lbox[3] = {(cuuint32_t)(kTiles[tile][0] + 2 * xo), (cuuint32_t)kTiles[tile][1] + 2, 1};
+    if (fn(reinterpret_cast<CUtensorMap*>(load_map), dt, 3, (void*)buf, ldims, strides, lbox, estr,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    cuuint64_t sdims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)Q};
+    cuuint32_t sbox[3] = {(cuuint32_t)kTiles[tile][0], (cuuint32_t)kTiles[tile][1], (cuuint32_t)Q};
+    return fn(reinterpret_cast<CUtensorMap*>(store_map), dt, 3, (char*)buf + g.at(0, 0) * es, sdims, strides, sbox, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 size_t tensor_map_bytes() { return sizeof(CUtensorMap); }
 
 template <int TX, int TY, int NT, int MODE, typename T, bool POLY = false>
-static cudaError_t launch_cfg(const void* map, TmaArgs ta, cudaStream_t s) {
+static cudaError_t launch_cfg(const void* const map[2], TmaArgs ta, cudaStream_t s) {
     using TT = TmaTile<TX, TY, T>;
     auto kern = step_tma_kernel<TX, TY, NT, MODE, T, POLY>;
-    constexpr int smem = TT::SMEM_BYTES + (MODE == 3 ? TT::H_BYTES : 0);
+    constexpr int smem = TT::SMEM_BYTES + (MODE == 3 ? StencilTile<TX, TY, NT>::BYTES : 0);
     static GridCache cache;
     int grid_max = 0;
     cudaError_t e = resident_grid(kern, NT, smem, cache, &grid_max);
     if (e != cudaSuccess) return e;
-    ta.ntx = (ta.a.g.nx + TX - 1) / TX;
-    ta.nty = (ta.a.g.ny + TY - 1) / TY;
+    ta.ntx = (ta.g.nx + TX - 1) / TX;
+    ta.nty = (ta.g.ny + TY - 1) / TY;
     const int ntiles = ta.ntx * ta.nty;
     const int grid = ntiles < grid_max ? ntiles : grid_max;
-    kern<<<grid, NT, smem, s>>>(*reinterpret_cast<const CUtensorMap*>(map), ta);
+    kern<<<grid, NT, smem, s>>>(*static_cast<const CUtensorMap*>(map[0]), *static_cast<const CUtensorMap*>(map[1]), ta);
     return cudaGetLastError();
 }
 
 template <int MODE, typename T>
-static cudaError_t launch_mode(const void* map, const TmaArgs& ta, int tile, cudaStream_t s) {
+static cudaError_t launch_mode(const void* const map[2], const TmaArgs& ta, int tile, cudaStream_t s) {
     switch (tile) {
         case 1: return launch_cfg<32, 32, 256, MODE, T>(map, ta, s);
         case 2: return launch_cfg<64, 8, 256, MODE, T>(map, ta, s);
@@ -271,7 +240,7 @@ static cudaError_t launch_mode(const void* map, const TmaArgs& ta, int tile, cud
 }
 
 template <typename T>
-static cudaError_t launch_type(const void* map, const TmaArgs& ta, int noise_mode, int tile, cudaStream_t s) {
+static cudaError_t launch_type(const void* const map[2], const TmaArgs& ta, int noise_mode, int tile, cudaStream_t s) {
     switch (noise_mode) {
         case 0: return launch_mode<0, T>(map, ta, tile, s);
         case 1: return launch_mode<1, T>(map, ta, tile, s);
@@ -283,25 +252,37 @@ static cudaError_t launch_type(const void* map, const TmaArgs& ta, int noise_mod
 
 // the double-well equation of state, FP32 storage: the default tile of each noise mode
 // (tma_default_tile(noise_mode, 0); the caller encodes the tensor maps for it)
-static cudaError_t launch_poly(const void* map, const TmaArgs& ta, int noise_mode, cudaStream_t s) {
+static cudaError_t launch_poly(const void* const map[2], const TmaArgs& ta, int noise_mode, cudaStream_t s) {
     switch (noise_mode) {
-        case 0: return launch_cfg<32, 32, 256, 0, float, true>(map, ta, s);
-        case 1: return launch_cfg<64, 16, 512, 1, float, true>(map, ta, s);
-        case 3: return launch_cfg<32, 16, 256, 3, float, true>(map, ta, s);
-        case 4: return launch_cfg<64, 16, 512, 4, float, true>(map, ta, s);
-        default: return launch_cfg<32, 16, 256, 2, float, true>(map, ta, s);
+        case 0: return launch_cfg<64, 8, 256, 0, float, true>(map, ta, s);
+        case 1: return launch_cfg<64, 8, 256, 1, float, true>(map, ta, s);
+        case 3: return launch_cfg<32, 16, 128, 3, float, true>(map, ta, s);
+        case 4: return launch_cfg<64, 8, 256, 4, float, true>(map, ta, s);
+        default: return launch_cfg<64, 8, 256, 2, float, true>(map, ta, s);
     }
 }
 
-cudaError_t launch_step_tma(const StepArgs& a, const void* src_map, int* err, int noise_mode, int tile, int fp16,
+cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* src_map, const void* dst_map, int* err, int noise_mode, int tile, int fp16,
                             cudaStream_t s, bool poly) {
     TmaArgs ta;
-    ta.a = a;
+    const double c = fp16 ? pair_scale<true>() : pair_scale<false>();
+    // the coefficients from FP64, rounded once
+    const double L[4] = {d.L44, d.L49, d.L94, d.L99}, s3[3] = {d.s5, d.s6, d.s7};
+    pair_coef(d.rho0, d.cs2m, d.kappa, d.lb, d.ls, d.lq, d.le, L, s3, c, &ta);
+    pair_stencil(d.sL, c, &ta);
+    pair_local(d.e2, d.e3, d.e4, d.cq, d.lu, c, &ta.loc);
+    ta.g = a.g;
+    ta.dst = a.dst;
+    ta.xi49 = a.xi49;
     ta.ntx = ta.nty = 0;
     ta.err = err;
-    if (poly) return fp16 ? cudaErrorInvalidValue : launch_poly(src_map, ta, noise_mode, s);
-    return fp16 ? launch_type<__half>(src_map, ta, noise_mode, tile, s)
-                : launch_type<float>(src_map, ta, noise_mode, tile, s);
+    ta.t_lo = a.t_lo;
+    ta.t_hi = a.t_hi;
+    ta.rk = a.rk;
+    const void* const map[2] = {src_map, dst_map};
+    if (poly) return fp16 ? cudaErrorInvalidValue : launch_poly(map, ta, noise_mode, s);
+    return fp16 ? launch_type<__half>(map, ta, noise_mode, tile, s)
+                : launch_type<float>(map, ta, noise_mode, tile, s);
 }
 
 }  // namespace lbf

@@ -7,6 +7,9 @@
 
 namespace lbf {
 
+// Shared memory of one CTA that steps TX x TY tiles: the stage (nine boxes of the tile being
+// loaded or pulled), the nine post-collision planes on their way out, the density tile with its
+// one-node ring, and the mbarrier.
 template <int TX, int TY, typename T>
 struct TmaTile {
     static constexpr int XO = Elem<T>::XO;                              // 16 bytes of elements
@@ -14,21 +17,18 @@ struct TmaTile {
     static constexpr int BH = TY + 2;                                   // box height
     static constexpr int PLANE_BYTES = BW * BH * (int)sizeof(T);
     static constexpr int PS = ((PLANE_BYTES + 127) / 128) * 128 / (int)sizeof(T);   // plane stride (elements)
-    static constexpr int STAGE = Q * PS;                                // elements per stage
-    static constexpr int STAGE_BYTES = STAGE * (int)sizeof(T);
-    static constexpr int RW = TX + 2, RH = TY + 2;                      // density tile + ring
-    static constexpr int SMEM_BYTES = 2 * STAGE_BYTES + RW * RH * 4 + 2 * 8;
+    static constexpr int STAGE_BYTES = Q * PS * (int)sizeof(T);
     static constexpr uint32_t TX_BYTES = Q * PLANE_BYTES;
-    // real-space correlated noise: h00, h10, h01, h11 (float2 each) of the tile's nodes and of
-    // the column left of it and the row below it, (TX + 1) x (TY + 1) nodes, after the mbarriers
-    static constexpr int HW = TX + 1;
-    static constexpr int HN = (TX + 1) * (TY + 1);
-    static constexpr int H_BYTES = 4 * HN * 8;
-    static constexpr int H_OFFSET = SMEM_BYTES;        // 16-byte aligned: RW, RH even
-    static_assert(H_OFFSET % 16 == 0, "H must be 16-byte aligned");
-    // whether H fits in the memory of one stage (FP32 storage): the engines put it in the
-    // stage just consumed and refill that stage after the collision pass
-    static constexpr bool H_IN_STAGE = H_BYTES <= STAGE_BYTES;
+    static constexpr int OUT = STAGE_BYTES;                             // [plane][TY][TX]: one box of the store map
+    static constexpr int OUT_BYTES = Q * TX * TY * (int)sizeof(T);
+    static_assert(OUT % 128 == 0 && OUT_BYTES % 128 == 0, "boxes start on 128 bytes");
+    // density tile + ring, node (lx, ly) at (ly + 1) RW + lx + 2: pairs of columns (lx even) on
+    // 8-byte boundaries
+    static constexpr int RW = TX + 4, RH = TY + 2;
+    static constexpr int RHO = OUT + OUT_BYTES;
+    static constexpr int BAR = RHO + RW * RH * 4;
+    static constexpr int SMEM_BYTES = BAR + 16;
+    static_assert(SMEM_BYTES % 16 == 0, "what follows is 16-byte aligned");
 };
 
 static __constant__ int kCYt[Q] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
@@ -78,6 +78,28 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// the box of shared memory at src to a tensor (part of the calling thread's current bulk group)
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(x), "r"(y), "r"(z), "r"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int x, int y, int z, int w) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(x), "r"(y), "r"(z), "r"(w), "r"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// the calling thread's committed stores have read their shared memory / are complete
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+// orders the calling thread's accesses to shared memory with those of later TMA operations
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w,
                                             uint32_t bar) {
     asm volatile(
@@ -104,65 +126,6 @@ __device__ __forceinline__ bool mbar_wait_bounded_ns(uint32_t bar, uint32_t pari
 
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
     return mbar_wait_bounded_ns(bar, parity, WAIT_LIMIT_NS);
-}
-
-// The nine pulled deviations of the node whose unshifted box index is b: plane i is read at
-// b - cx_i (its y shift is already in the box origin).
-template <int PS, typename T, bool GF = false>
-__device__ __forceinline__ void load9_ps(const T* S, int b, float f[Q]) {
-    auto ld = [](T v, int i) -> float {
-        if constexpr (GF) return Elem<T>::load_g(v);
-        else return Elem<T>::load(v, i);
-    };
-    f[0] = ld(S[b], 0);
-    f[1] = ld(S[PS + b - 1], 1);
-    f[2] = ld(S[2 * PS + b], 2);
-    f[3] = ld(S[3 * PS + b + 1], 3);
-    f[4] = ld(S[4 * PS + b], 4);
-    f[5] = ld(S[5 * PS + b - 1], 5);
-    f[6] = ld(S[6 * PS + b + 1], 6);
-    f[7] = ld(S[7 * PS + b + 1], 7);
-    f[8] = ld(S[8 * PS + b - 1], 8);
-}
-
-// Real-space correlated noise of a tile (LB_NOISE_FULL_RS): the contributions h_d(q) of a
-// node q of the tile, or of the column left of it / row below it (local coordinates -1),
-// go to H[d][(ly + 1) * HW + lx + 1]; the (xi_4, xi_9) of a tile node are then
-// h00(r) + h10(r - e_x) + h01(r - e_y) + h11(r - e_x - e_y).
-template <int HW, typename Args>
-__device__ __forceinline__ void stencil_store(const Args& a, float2* H, int HN, int lx, int ly, uint32_t node) {
-    float h[8];
-    stencil_h(a, node, h);
-    const int q = (ly + 1) * HW + lx + 1;
-    H[q] = make_float2(h[0], h[1]);
-    H[HN + q] = make_float2(h[2], h[3]);
-    H[2 * HN + q] = make_float2(h[4], h[5]);
-    H[3 * HN + q] = make_float2(h[6], h[7]);
-}
-
-// the halo nodes of the tile at (x0, y0): j in [0, TY] -> column x0 - 1, rows y0 - 1 ..
-// y0 + TY - 1; j in (TY, TX + TY] -> row y0 - 1, columns x0 .. x0 + TX - 1 (periodic; nodes
-// past a ragged edge are skipped, no tile node reads them).  They go to the last threads of
-// the block, which form no density-ring node, so the work before the tile's barrier evens out.
-template <int TX, int TY, int HW, typename Args>
-__device__ __forceinline__ void stencil_halo(const Args& a, float2* H, int HN, int x0, int y0, int nx, int ny,
-                                             int tid, int nthreads) {
-    for (int j = nthreads - 1 - tid; j < TX + TY + 1; j += nthreads) {
-        int lx, ly;
-        if (j <= TY) { lx = -1; ly = j - 1; }
-        else { lx = j - (TY + 1); ly = -1; }
-        int gx = x0 + lx, gy = y0 + ly;
-        if (gx < 0) gx += nx;
-        if (gy < 0) gy += ny;
-        if (gx < nx && gy < ny) stencil_store<HW>(a, H, HN, lx, ly, (uint32_t)gy * (uint32_t)nx + (uint32_t)gx);
-    }
-}
-
-template <int HW>
-__device__ __forceinline__ float2 stencil_xi(const float2* H, int HN, int lx, int ly) {
-    const int q = (ly + 1) * HW + lx + 1;
-    const float2 a = H[q], b = H[HN + q - 1], c = H[2 * HN + q - HW], d = H[3 * HN + q - HW - 1];
-    return make_float2((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
 }
 
 }  // namespace lbf
