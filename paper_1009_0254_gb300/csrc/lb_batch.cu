@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    grid_wait();
+    grid_next();
     const long long K = __ldcg(p.kstep);
     const int par = (int)(K & 1);
 
@@ -400,9 +402,9 @@ static cudaError_t launch_ensemble_t(const EnsParams& p, cudaStream_t s) {
     cudaError_t e = p.rs ? ensemble_grid<TX, TY, NT, true>(&grid) : ensemble_grid<TX, TY, NT, false>(&grid);
     if (e != cudaSuccess) return e;
     const int blocks = std::max(1, std::min(p.ntiles, grid));
-    if (p.rs) step_ensemble_kernel<TX, TY, NT, true><<<blocks, NT, ensemble_smem<TX, TY, NT, true>(), s>>>(p);
-    else step_ensemble_kernel<TX, TY, NT, false><<<blocks, NT, ensemble_smem<TX, TY, NT, false>(), s>>>(p);
-    return cudaGetLastError();
+    if (p.rs)
+        return launch_chained(step_ensemble_kernel<TX, TY, NT, true>, blocks, NT, ensemble_smem<TX, TY, NT, true>(), s, p);
+    return launch_chained(step_ensemble_kernel<TX, TY, NT, false>, blocks, NT, ensemble_smem<TX, TY, NT, false>(), s, p);
 }
 
 static cudaError_t launch_ensemble(int tile, const EnsParams& p, cudaStream_t s) {

@@ -414,6 +414,30 @@ cudaError_t resident_grid(K kern, int threads, int smem, GridCache& c, int* grid
     return cudaSuccess;
 }
 
+// Step kernels are launched so that the next launch of their stream may start its CTAs, as far as
+// room is left, before the last one has ended: grid_wait() then holds them until every earlier
+// kernel of the stream has completed and its writes are visible (no global memory is touched before
+// it), and grid_next() after it lets the launch that follows start in turn.  A launch that neither
+// asks for this nor follows one that does behaves as always.  What it takes away is the launch
+// latency between dependent steps, most of a step on lattices below 512^2.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), int grid, int threads, int smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = (size_t)smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
 }  // namespace lbf
 
 // Launchers implemented in the .cu files (host side).

@@ -111,6 +111,8 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    grid_wait();
+    grid_next();
     const long long K = __ldcg(p.kstep);
 
     // thread 0: the record of a tile, and its slot's maps for this step, their descriptors made
@@ -781,8 +783,8 @@ bool issue_chunk(lb_server* s) {
                 s->d_full[c] + gr.off, s->d_desc, gr.nx, gr.ny, tb2.twx,
                 (float)(1.0 / std::sqrt((double)gr.nx * gr.ny)));
         }
-        if (rs) step_serve_kernel<SV_TX, SV_TY, SV_NT, true><<<grid, SV_NT, serve_smem<true>(), s->stream>>>(p);
-        else step_serve_kernel<SV_TX, SV_TY, SV_NT, false><<<grid, SV_NT, serve_smem<false>(), s->stream>>>(p);
+        if (rs) SCK(s, launch_chained(step_serve_kernel<SV_TX, SV_TY, SV_NT, true>, grid, SV_NT, serve_smem<true>(), s->stream, p));
+        else SCK(s, launch_chained(step_serve_kernel<SV_TX, SV_TY, SV_NT, false>, grid, SV_NT, serve_smem<false>(), s->stream, p));
     }
     SCK(s, cudaGetLastError());
     s->K += G;

@@ -81,6 +81,8 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>())
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&smap)) : "memory");
     }
     __syncthreads();
+    grid_wait();
+    grid_next();
 
     // the nine boxes of the tile in column col, row row of the tiling
     auto load = [&](int col, int row) {
@@ -224,8 +226,8 @@ static cudaError_t launch_cfg(const void* const map[2], TmaArgs ta, cudaStream_t
     ta.nty = (ta.g.ny + TY - 1) / TY;
     const int ntiles = ta.ntx * ta.nty;
     const int grid = ntiles < grid_max ? ntiles : grid_max;
-    kern<<<grid, NT, smem, s>>>(*static_cast<const CUtensorMap*>(map[0]), *static_cast<const CUtensorMap*>(map[1]), ta);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NT, smem, s, *static_cast<const CUtensorMap*>(map[0]),
+                          *static_cast<const CUtensorMap*>(map[1]), ta);
 }
 
 template <int MODE, typename T>
