@@ -10,6 +10,7 @@
 // with a twiddle table exp(-2 pi i q/n) computed on the host in FP64 (one read per
 // butterfly, its powers formed on the fly).
 #include <algorithm>
+#include <utility>
 
 #include "lb_fft_core.cuh"
 #include "lb_internal.cuh"
@@ -24,6 +25,8 @@ __device__ __forceinline__ int ilog2(int n) { return 31 - __clz(n); }
 // more points read and write global memory in the first and last stage directly.
 __global__ void __launch_bounds__(1024) fft_rows_kernel(float2* data, int nx, int sign, const float2* __restrict__ twx, float scale) {
     extern __shared__ float2 sm[];
+    grid_wait();
+    grid_next();
     const int log2n = ilog2(nx);
     float2* rowp = data + (long long)blockIdx.x * nx;
     if (nx >= 256) {
@@ -46,11 +49,15 @@ __global__ void __launch_bounds__(1024) fft_rows_kernel(float2* data, int nx, in
 template <bool PERM>
 __global__ void __launch_bounds__(1024) noise_cols_kernel(float2* out, NoiseGenArgs ga, int count,
                                                           const float2* __restrict__ twy) {
+    grid_wait();
+    grid_next();
     noise_cols_block<PERM>(out, ga, count, blockIdx.x, twy);
 }
 
 __global__ void __launch_bounds__(1024) noise_rows_kernel(const float2* __restrict__ h, float2* xi, int nx, int ny,
                                                           int count, const float2* __restrict__ twx, float scale) {
+    grid_wait();
+    grid_next();
     noise_rows_gather(h, xi, nx, count, (int)blockIdx.x, twx, scale);
 }
 
@@ -60,6 +67,8 @@ __global__ void __launch_bounds__(512) fft_rows_kernel_d(double2* data, int nx, 
     extern __shared__ __align__(16) unsigned char rows_smem_d[];
     double2* sm = reinterpret_cast<double2*>(rows_smem_d);
     double2* rowp = data + (long long)blockIdx.x * nx;
+    grid_wait();
+    grid_next();
     for (int j = threadIdx.x; j < nx; j += blockDim.x) sm[fpad(j)] = rowp[j];
     stockham_fft(sm, nx, ilog2(nx), 1, sign, twx);
     for (int j = threadIdx.x; j < nx; j += blockDim.x) {
@@ -70,6 +79,8 @@ __global__ void __launch_bounds__(512) fft_rows_kernel_d(double2* data, int nx, 
 
 __global__ void __launch_bounds__(512) noise_cols_kernel_d(double2* out, NoiseGenArgsD ga, int count,
                                                             const double2* __restrict__ twy) {
+    grid_wait();
+    grid_next();
     noise_cols_block<false>(out, ga, count, blockIdx.x, twy);
 }
 
@@ -77,6 +88,8 @@ __global__ void __launch_bounds__(512) noise_cols_kernel_d(double2* out, NoiseGe
 __global__ void __launch_bounds__(1024) fft_cols_kernel(float2* data, int nx, int ny, int count, int sign,
                                 const float2* __restrict__ twy, float scale) {
     extern __shared__ float2 sm[];
+    grid_wait();
+    grid_next();
     const int log2n = ilog2(ny);
     const int xs = blockIdx.x * count;
     const int total = ny * count;
@@ -110,23 +123,35 @@ static int col_strip(int nx, int ny) {
     return c;
 }
 
+// Strip width of the correlated noise's column pass: on small lattices narrower (a block pairs at
+// least two columns), until the pass has a CTA for nearly every SM.  A CTA's columns are synthesised
+// one wavevector a thread and turn, so 64^2 in 4 CTAs took 8 turns of 64 threads where 32 CTAs take 2.
+static int noise_strip(int nx, int c) {
+    while (c > 2 && nx / c < 128) c >>= 1;
+    return c;
+}
+
+// launch of a transform kernel (its dynamic shared-memory limit raised where it asks for more than
+// the 48 KB that every kernel may use)
+template <typename... P, typename... A>
+static cudaError_t launch_fft(void (*kern)(P...), int grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_chained(kern, dim3(grid), dim3(threads), smem, s, std::forward<A>(args)...);
+}
+
 static cudaError_t rows_pass(float2* data, int nx, int ny, int sign, const float2* twx, float scale,
                              cudaStream_t s) {
-    const size_t smem = fft_smem_bytes(nx, 1);
-    cudaError_t e = cudaFuncSetAttribute(fft_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    fft_rows_kernel<<<ny, fft_threads(nx, 1), smem, s>>>(data, nx, sign, twx, scale);
-    return cudaGetLastError();
+    return launch_fft(fft_rows_kernel, ny, fft_threads(nx, 1), fft_smem_bytes(nx, 1), s, data, nx, sign, twx, scale);
 }
 
 static cudaError_t cols_pass(float2* data, int nx, int ny, int sign, const float2* twy, float scale,
                              cudaStream_t s) {
     const int c = col_strip(nx, ny);
-    const size_t smem = fft_smem_bytes(ny, c);
-    cudaError_t e = cudaFuncSetAttribute(fft_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    fft_cols_kernel<<<nx / c, fft_threads(ny, c), smem, s>>>(data, nx, ny, c, sign, twy, scale);
-    return cudaGetLastError();
+    return launch_fft(fft_cols_kernel, nx / c, fft_threads(ny, c), fft_smem_bytes(ny, c), s, data, nx, ny, c, sign, twy,
+                      scale);
 }
 
 cudaError_t launch_fft2d(float2* data, int nx, int ny, int sign, const float2* twx, const float2* twy,
@@ -143,28 +168,19 @@ cudaError_t launch_noise49(float2* buf, float2* scratch, const NoiseGenArgs& ga,
     // Rows of 256 points and more go through the column-permuted scratch (whole 32-byte
     // sectors per write, rows gathered back in the first stage of the row transform:
     // 219 -> 171 us at 4096^2, 118 -> 115 us a step at 2048^2); shorter rows stay in place.
-    const int c = col_strip(ga.nx, ga.ny);
+    const int c = noise_strip(ga.nx, col_strip(ga.nx, ga.ny));
     if (c < 2) return cudaErrorInvalidValue;
-    const bool perm = ga.nx >= 256;
     const size_t smem = fft_smem_bytes(ga.ny, c);
     const float scale = (float)(1.0 / sqrt((double)ga.nx * (double)ga.ny));
     cudaError_t e;
-    if (!perm) {
-        e = cudaFuncSetAttribute(noise_cols_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        noise_cols_kernel<false><<<ga.nx / c, fft_threads(ga.ny, c), smem, s>>>(buf, ga, c, twy);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return rows_pass(buf, ga.nx, ga.ny, -1, twx, scale, s);
+    if (ga.nx < 256) {
+        e = launch_fft(noise_cols_kernel<false>, ga.nx / c, fft_threads(ga.ny, c), smem, s, buf, ga, c, twy);
+        return e != cudaSuccess ? e : rows_pass(buf, ga.nx, ga.ny, -1, twx, scale, s);
     }
-    e = cudaFuncSetAttribute(noise_cols_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = launch_fft(noise_cols_kernel<true>, ga.nx / c, fft_threads(ga.ny, c), smem, s, scratch, ga, c, twy);
     if (e != cudaSuccess) return e;
-    noise_cols_kernel<true><<<ga.nx / c, fft_threads(ga.ny, c), smem, s>>>(scratch, ga, c, twy);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t rsm = fft_smem_bytes(ga.nx, 1);
-    e = cudaFuncSetAttribute(noise_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
-    if (e != cudaSuccess) return e;
-    noise_rows_kernel<<<ga.ny, fft_threads(ga.nx, 1), rsm, s>>>(scratch, buf, ga.nx, ga.ny, c, twx, scale);
-    return cudaGetLastError();
+    return launch_fft(noise_rows_kernel, ga.ny, fft_threads(ga.nx, 1), fft_smem_bytes(ga.nx, 1), s, scratch, buf, ga.nx,
+                      ga.ny, c, twx, scale);
 }
 
 int noise_strip_d(int nx, int ny) {
@@ -175,19 +191,15 @@ int noise_strip_d(int nx, int ny) {
 
 cudaError_t launch_noise49_d(double2* buf, const NoiseGenArgsD& ga, const double2* twx, const double2* twy,
                              cudaStream_t s) {
-    const int c = noise_strip_d(ga.nx, ga.ny);
+    const int c = noise_strip(ga.nx, noise_strip_d(ga.nx, ga.ny));
     if (c < 2) return cudaErrorInvalidValue;
-    const size_t smem = fft_smem_bytes(ga.ny, c, 16);
-    cudaError_t e = cudaFuncSetAttribute(noise_cols_kernel_d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // a thread per radix-4 butterfly or per pair of wavevectors, whichever is more (both at most 512)
+    auto threads = [](int n) { return n < 32 ? 32 : (n > 512 ? 512 : n); };
+    const cudaError_t e = launch_fft(noise_cols_kernel_d, ga.nx / c, threads(ga.ny * c / 2), fft_smem_bytes(ga.ny, c, 16), s,
+                                     buf, ga, c, twy);
     if (e != cudaSuccess) return e;
-    noise_cols_kernel_d<<<ga.nx / c, fft_threads(ga.ny, c), smem, s>>>(buf, ga, c, twy);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t rsm = fft_smem_bytes(ga.nx, 1, 16);
-    e = cudaFuncSetAttribute(fft_rows_kernel_d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
-    if (e != cudaSuccess) return e;
-    fft_rows_kernel_d<<<ga.ny, fft_threads(ga.nx, 1), rsm, s>>>(buf, ga.nx, -1, twx,
-                                                                1.0 / sqrt((double)ga.nx * (double)ga.ny));
-    return cudaGetLastError();
+    return launch_fft(fft_rows_kernel_d, ga.ny, threads(ga.nx / 4), fft_smem_bytes(ga.nx, 1, 16), s, buf, ga.nx, -1, twx,
+                      1.0 / sqrt((double)ga.nx * (double)ga.ny));
 }
 
 // --- sampled spectra ---------------------------------------------------------------

@@ -155,18 +155,26 @@ __device__ __forceinline__ void stockham_stage(C* s, int n, int count, int lc, i
     __syncthreads();
 }
 
+// Largest radix of a transform's stages.  FP32: 16 (fewest passes over shared memory).  FP64: 4, at the
+// same number of operations: four times as many threads share a transform, whose time is the latency of
+// its chain of FP64 operations, 16 cycles each at best (64-point rows: 4 threads and 350 operations each
+// in the first radix-16 stage, 16 threads and 46 a stage with radix 4).
+template <typename C>
+__host__ __device__ constexpr int fft_log2_radix() { return sizeof(C) == 16 ? 2 : 4; }
+
 // Full transform of `count` interleaved sequences of length n = 2^log2n (n >= 2) already in
 // shared memory; tw[q] = exp(-2 pi i q / n), q < n.  Needs blockDim.x >= max(1, n/16) * count.
 template <typename C>
 __device__ __forceinline__ void stockham_fft(C* s, int n, int log2n, int count, int sign,
                                              const C* __restrict__ tw) {
     const int lc = 31 - __clz(count);
+    constexpr int LR = fft_log2_radix<C>();
     int Ns = 1, left = log2n;
     __syncthreads();
-    while (left >= 4) {
-        stockham_stage<16>(s, n, count, lc, Ns, sign, tw);
-        Ns <<= 4;
-        left -= 4;
+    while (left >= LR) {
+        stockham_stage<(1 << LR)>(s, n, count, lc, Ns, sign, tw);
+        Ns <<= LR;
+        left -= LR;
     }
     if (left == 3) stockham_stage<8>(s, n, count, lc, Ns, sign, tw);
     else if (left == 2) stockham_stage<4>(s, n, count, lc, Ns, sign, tw);
@@ -262,12 +270,13 @@ template <typename C, typename Store>
 __device__ __forceinline__ void stockham_fft_out(C* s, int n, int log2n, int count, int sign,
                                                  const C* __restrict__ tw, Store store) {
     const int lc = 31 - __clz(count);
+    constexpr int LR = fft_log2_radix<C>();
     int Ns = 1, left = log2n;
     __syncthreads();
-    while (left > 4) {
-        stockham_stage<16>(s, n, count, lc, Ns, sign, tw);
-        Ns <<= 4;
-        left -= 4;
+    while (left > LR) {
+        stockham_stage<(1 << LR)>(s, n, count, lc, Ns, sign, tw);
+        Ns <<= LR;
+        left -= LR;
     }
     if (left == 4) stockham_last<16>(s, n, count, lc, sign, tw, store);
     else if (left == 3) stockham_last<8>(s, n, count, lc, sign, tw, store);

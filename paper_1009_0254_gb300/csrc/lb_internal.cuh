@@ -232,14 +232,14 @@ __device__ __forceinline__ float2 gauss_pair(uint32_t w) {
     return make_float2(-r * __cosf(th), -r * __sinf(th));
 }
 
-// The same pair in FP64 (storage LB_FP64): IEEE log, sqrt and sincos, the form of the
-// definition itself.
+// The same pair in FP64 (storage LB_FP64): IEEE log and sqrt, sine and cosine of pi 2 u2 (2 u2 is
+// exact, so no rounding of the angle and no range reduction by pi).
 __device__ __forceinline__ double2 gauss_pair_d(uint32_t w) {
     const double u1 = ((double)(w >> 12) + 0.5) * (1.0 / 1048576.0);
     const double u2 = ((double)(w & 0xfffu) + 0.5) * (1.0 / 4096.0);
     const double r = sqrt(-2.0 * log(u1));
     double sn, cs;
-    sincos(6.283185307179586476925286766559 * u2, &sn, &cs);
+    sincospi(2.0 * u2, &sn, &cs);
     return make_double2(r * cs, r * sn);
 }
 
@@ -424,11 +424,11 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 __device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kern)(P...), int grid, int threads, int smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t s, A&&... args) {
     cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(grid);
-    c.blockDim = dim3(threads);
-    c.dynamicSmemBytes = (size_t)smem;
+    c.gridDim = grid;
+    c.blockDim = threads;
+    c.dynamicSmemBytes = smem;
     c.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -71,6 +71,8 @@ __global__ void __launch_bounds__(BX * BY) step_kernel(const StepArgsT<typename 
     const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
     const int x = x0 + tx, y = y0 + ty;
     const bool own = (x < g.nx) && (y < g.ny);
+    grid_wait();
+    grid_next();
 
     // 1. density on the tile (plus the first column/row past a ragged edge)
     R f[Q];
@@ -140,36 +142,44 @@ __global__ void __launch_bounds__(BX * BY) step_kernel(const StepArgsT<typename 
     store9(static_cast<T*>(a.dst), P, g, x, y, o);
 }
 
-template <typename T, bool POLY>
-static void launch_p(const StepArgsT<typename Arith<T>::type>& a, int noise_mode, cudaStream_t s) {
-    constexpr int BX = 32, BY = 16;
-    dim3 block(BX, BY);
-    dim3 grid((a.g.nx + BX - 1) / BX, (a.g.ny + BY - 1) / BY);
+template <typename T, bool POLY, int BX, int BY>
+static cudaError_t launch_p(const StepArgsT<typename Arith<T>::type>& a, int noise_mode, cudaStream_t s) {
+    const dim3 block(BX, BY), grid((a.g.nx + BX - 1) / BX, (a.g.ny + BY - 1) / BY);
     switch (noise_mode) {
-        case 0: step_kernel<BX, BY, 0, T, POLY><<<grid, block, 0, s>>>(a); break;
-        case 1: step_kernel<BX, BY, 1, T, POLY><<<grid, block, 0, s>>>(a); break;
-        case 3: step_kernel<BX, BY, 3, T, POLY><<<grid, block, 0, s>>>(a); break;
-        case 4: step_kernel<BX, BY, 4, T, POLY><<<grid, block, 0, s>>>(a); break;
-        default: step_kernel<BX, BY, 2, T, POLY><<<grid, block, 0, s>>>(a); break;
+        case 0: return launch_chained(step_kernel<BX, BY, 0, T, POLY>, grid, block, 0, s, a);
+        case 1: return launch_chained(step_kernel<BX, BY, 1, T, POLY>, grid, block, 0, s, a);
+        case 3: return launch_chained(step_kernel<BX, BY, 3, T, POLY>, grid, block, 0, s, a);
+        case 4: return launch_chained(step_kernel<BX, BY, 4, T, POLY>, grid, block, 0, s, a);
+        default: return launch_chained(step_kernel<BX, BY, 2, T, POLY>, grid, block, 0, s, a);
     }
 }
 
 // the double-well equation of state (a.eos) is a separate instantiation
-template <typename T>
-static void launch_t(const StepArgsT<typename Arith<T>::type>& a, int noise_mode, cudaStream_t s) {
-    if (a.eos) launch_p<T, true>(a, noise_mode, s);
-    else launch_p<T, false>(a, noise_mode, s);
+template <typename T, int BX, int BY>
+static cudaError_t launch_t(const StepArgsT<typename Arith<T>::type>& a, int noise_mode, cudaStream_t s) {
+    return a.eos ? launch_p<T, true, BX, BY>(a, noise_mode, s) : launch_p<T, false, BX, BY>(a, noise_mode, s);
 }
 
 cudaError_t launch_step_simple(const StepArgs& a, int noise_mode, int fp16, cudaStream_t s) {
-    if (fp16) launch_t<__half>(a, noise_mode, s);
-    else launch_t<float>(a, noise_mode, s);
-    return cudaGetLastError();
+    return fp16 ? launch_t<__half, 32, 16>(a, noise_mode, s) : launch_t<float, 32, 16>(a, noise_mode, s);
 }
 
+// FP64: an SM issues two FP64 operations a clock, and a node needs some 150 of them, plus 115 for each
+// of its Box-Muller pairs (logarithm, root, sine and cosine), so a 32 x 16 tile takes its SM 46 us and
+// what counts is that every SM has its share.  The tile height (16, 4 or 1 rows) of the least work on
+// the busiest SM is taken, the density ring and, with the real-space noise, the halo's draws counted.
+// Uncorrelated noise, us a step, 32 x 16 tiles alone and by this rule: 64^2 56 and 16, 512^2 212 and 188.
 cudaError_t launch_step_simple_d(const StepArgsD& a, int noise_mode, cudaStream_t s) {
-    launch_t<double>(a, noise_mode, s);
-    return cudaGetLastError();
+    const long long tx = (a.g.nx + 31) / 32;
+    const int pairs = noise_mode == 0 ? 0 : (noise_mode == 2 ? 2 : (noise_mode == 3 ? 6 : 3));
+    auto work = [&](int by) {
+        const long long ctas = tx * ((a.g.ny + by - 1) / by), turns = (ctas + 151) / 152;
+        return turns * (32 * by * (150 + 115 * pairs) + (68 + 2 * by) * 8 + (noise_mode == 3 ? (33 + by) * 4 * 115 : 0));
+    };
+    const long long w16 = work(16), w4 = work(4), w1 = work(1);
+    if (w16 <= w4 && w16 <= w1) return launch_t<double, 32, 16>(a, noise_mode, s);
+    if (w4 <= w1) return launch_t<double, 32, 4>(a, noise_mode, s);
+    return launch_t<double, 32, 1>(a, noise_mode, s);
 }
 
 }  // namespace lbf
