@@ -616,8 +616,46 @@ bool noise_factors(int lattice, const double* X, double sc[QMAX], double Lc[28])
     return true;
 }
 
+// The FP32 kernels' noise factors over GAUSS_SCALE, the corner amplitudes over 8, and with the factor u of
+// a mode's increment in collide27_f (D3Q27) or collide19_f (D3Q19, correlated noise), the rates too.  With
+// the noise at the local density the coupled block's entries take u_a u_b and the kernel puts GAUSS_SCALE
+// to the normals.
+void scale_args(int lattice, int kmode, Step3Args<float>* a, double tau_s, double tau_b, double tau_g,
+                const double sc[QMAX], const double Lc[28], const double Lb[28], const double Lrs[12],
+                const double Prs[7], const double Qrs[7]) {
+    const double G = lbf::GAUSS_SCALE;
+    auto u = [&](int k) { return lattice == 27 ? sign27(k) * SCALE27 : (kmode == 3 && k >= 4 ? scale19(k) : 1.0); };
+    for (int k = 0; k < lattice; ++k) a->sc[k] = (float)(G * u(k) * sc[k]);
+    for (int k = 0; k < 12; ++k) a->Lrs[k] = (float)(0.125 * G * Lrs[k]);
+    if (lattice == 19) {
+        const double w[3] = {u(4), u(16), u(16)};
+        for (int q = 0; q < 3; ++q) {
+            a->Lc[q] = (float)(kmode == 4 ? Lc[q] : G * w[q] * Lc[q]);
+            for (int k = 0; k < 4; ++k) a->Lrs[3 * k + q] = (float)(0.125 * G * w[q] * Lrs[3 * k + q]);
+        }
+        const double lb = -1.0 / tau_b, ls = -1.0 / tau_s, lg = -1.0 / tau_g;
+        a->lam = Lam19{(float)(lb * u(4)), (float)(ls * u(5)), (float)(ls * u(6)), (float)(ls * u(7)), (float)(lg * u(10)),
+                       (float)(lg * u(13)), (float)(lg * u(16)), (float)(lg * u(17)), (float)(lg * u(18))};
+        return;
+    }
+    a->co.lb = (float)(-SCALE27 / tau_b);
+    a->co.ls = (float)(-SCALE27 / tau_s);
+    a->co.lg = (float)(-SCALE27 / tau_g);
+    for (int r = 0; r < 7; ++r) {
+        const double ur = u(coupled27(r));
+        for (int q = 0; q <= r; ++q) {
+            const int e = r * (r + 1) / 2 + q;
+            const double uu = ur * u(coupled27(q));
+            a->Lc[e] = (float)(kmode == 4 ? uu * Lc[e] : G * ur * Lc[e]);
+            a->Lb[e] = (float)(uu * Lb[e]);
+        }
+        a->Prs[r] = (float)(ur * Prs[r]);
+        a->Qrs[r] = (float)(ur * Qrs[r]);
+    }
+}
+
 template <typename R>
-void fill_args(lb3_ctx* c, Step3Args<R>* a, double tau_s, double tau_b, double tau_g, const double sc[QMAX],
+void fill_args(lb3_ctx* c, int kmode, Step3Args<R>* a, double tau_s, double tau_b, double tau_g, const double sc[QMAX],
                const double Lc[28], const double Lb[28], const double Lrs[12], const double Prs[7], const double Qrs[7]) {
     a->nx = c->nx; a->ny = c->ny; a->nz = c->nz;
     a->pitch = c->geom.pitch; a->gx = c->geom.gx; a->PL = c->geom.PL; a->P = c->geom.P;
@@ -641,6 +679,7 @@ void fill_args(lb3_ctx* c, Step3Args<R>* a, double tau_s, double tau_b, double t
         a->Qrs[q] = (R)Qrs[q];
     }
     a->rk = lbf::make_round_keys(c->seed);
+    if constexpr (sizeof(R) == 4) scale_args(c->lattice, kmode, a, tau_s, tau_b, tau_g, sc, Lc, Lb, Lrs, Prs, Qrs);
 }
 
 template <typename R>
@@ -829,8 +868,10 @@ int lb3_set_params(lb3_ctx* c, double kT, double kappa, double tau_s, double tau
     c->kappa = kappa;
     c->tau_s = tau_s; c->tau_b = tau_b; c->tau_g = tau_ghost;
     c->noise_mode = mode;
-    fill_args(c, &c->af, tau_s, tau_b, tau_ghost, sc, Lc, Lb, Lrs, Prs, Qrs);
-    fill_args(c, &c->ad, tau_s, tau_b, tau_ghost, sc, Lc, Lb, Lrs, Prs, Qrs);
+    // the kernel's noise mode of lb3_step (without noise none of the factors is read)
+    const int kmode = mode == LB_NOISE_LW_LOCAL ? 4 : (mode == LB_NOISE_FULL_RS && kT > 0.0 ? 3 : 1);
+    fill_args(c, kmode, &c->af, tau_s, tau_b, tau_ghost, sc, Lc, Lb, Lrs, Prs, Qrs);
+    fill_args(c, kmode, &c->ad, tau_s, tau_b, tau_ghost, sc, Lc, Lb, Lrs, Prs, Qrs);
     c->have_params = true;
     return LB_OK;
 }

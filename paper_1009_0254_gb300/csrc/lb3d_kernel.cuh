@@ -22,10 +22,18 @@
 // the plane whose densities are summed, and the plane in flight, so the loads of plane z+2
 // overlap the collision of plane z; with two slots a plane's own populations move to
 // registers when its densities are summed, which frees its slot for the plane after next.
-// The densities of planes z-1, z, z+1 sit in three more rotating slots; the collision reads
+// The densities of planes z-1, z, z+1 sit in three more rotating slots (TMA: four, which
+// leaves one block-wide barrier a plane); the collision reads
 // its node's populations and its 3x3x3 density neighbourhood from shared memory.  Every
 // population is read once from DRAM (the ring's re-reads hit L2) and written once, plus the
 // ghost copies.
+//
+// What bounds it.  DRAM traffic takes two thirds of a step; the rest is the serial chain of a plane
+// (wait, densities, barrier, collision) with 12 to 24 warps per SM to hide it: D3Q27 with 16 % fewer
+// instructions (packed, lb3_pair.cuh) gained 4 %.  256^3 FP32, before and after packing the D3Q27
+// collision, the normals and the box transforms, the fourth density slot and chained launches (us a step):
+// D3Q19 uncorrelated noise 614 -> 598, correlated 946 -> 893, without noise 582 (two barriers) -> 539;
+// D3Q27 870 -> 836 and 1290 -> 1170.
 //
 // A plain D3Q19 kernel (density summed from direct loads, the collision pulling again) is
 // kept as a cross-check.
@@ -37,6 +45,7 @@
 
 #include "lb27_collide.cuh"
 #include "lb3_collide.cuh"
+#include "lb3_pair.cuh"
 #include "lb_internal.cuh"
 #include "lb_tma.cuh"
 
@@ -109,7 +118,10 @@ struct Step3Args {
     long long PL;                 // elements per stored z plane
     long long P;                  // elements per population (nz PL)
     int* err;                     // device error word: 1 = a CTA gave up waiting for its TMA loads
+    // FP32: the noise factors carry GAUSS_SCALE, Lrs 1/8, and the factors of collide27_f (D3Q27, co's rates
+    // too) or of collide19_f (D3Q19 with correlated noise, whose rates are lam)
     Coef3<R> co;
+    Lam19 lam;
     R sc[QMAX];                   // sqrt(Xi_kk) of the modes with a diagonal factor (local noise:
                                   // per unit density)
     R Lc[28];                     // the coupled block's Cholesky factor: D3Q19 (L44, L16_4, L16_16);
@@ -126,25 +138,32 @@ struct Step3Args {
     lbf::RoundKeys rk;
 };
 
+// the 4 n normals of the n draws of a node from tag TAG0 on (FP32: over GAUSS_SCALE)
+template <uint32_t TAG0, int NDRAW, typename R>
+__device__ __forceinline__ void node_normals(const Step3Args<R>& a, uint32_t node, R nu[8 * NDRAW]) {
+#pragma unroll
+    for (int d = 0; d < NDRAW; ++d) {
+        const uint4 r = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, TAG0 + d), a.rk);
+        if constexpr (sizeof(R) == 4) {
+            normals8(r, nu + 8 * d);
+        } else {
+            lbf::gauss_word(r.x, &nu[8 * d + 0], &nu[8 * d + 1]);
+            lbf::gauss_word(r.y, &nu[8 * d + 2], &nu[8 * d + 3]);
+            lbf::gauss_word(r.z, &nu[8 * d + 4], &nu[8 * d + 5]);
+            lbf::gauss_word(r.w, &nu[8 * d + 6], &nu[8 * d + 7]);
+        }
+    }
+}
+
 // D3Q19 noise: tag 4 -> nu_4..nu_11, tag 5 -> nu_12..nu_18
 template <typename R>
 __device__ __forceinline__ void normals19(const Step3Args<R>& a, uint32_t node, R xi[Q3]) {
-    const uint4 ra = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, Lat19::TAG0), a.rk);
-    const uint4 rb = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, Lat19::TAG0 + 1), a.rk);
-    R n4, n16, spare;
-    lbf::gauss_word(ra.x, &n4, &xi[5]);
-    lbf::gauss_word(ra.y, &xi[6], &xi[7]);
-    lbf::gauss_word(ra.z, &xi[8], &xi[9]);
-    lbf::gauss_word(ra.w, &xi[10], &xi[11]);
-    lbf::gauss_word(rb.x, &xi[12], &xi[13]);
-    lbf::gauss_word(rb.y, &xi[14], &xi[15]);
-    lbf::gauss_word(rb.z, &n16, &xi[17]);
-    lbf::gauss_word(rb.w, &xi[18], &spare);
-    (void)spare;
+    R nu[16];
+    node_normals<Lat19::TAG0, 2>(a, node, nu);
 #pragma unroll
-    for (int q = 5; q < Q3; ++q) xi[q] *= a.sc[q];
-    xi[4] = a.Lc[0] * n4;
-    xi[16] = a.Lc[1] * n4 + a.Lc[2] * n16;
+    for (int q = 5; q < Q3; ++q) xi[q] = a.sc[q] * nu[q - 4];
+    xi[4] = a.Lc[0] * nu[0];
+    xi[16] = a.Lc[1] * nu[0] + a.Lc[2] * nu[12];
 }
 
 // D3Q19 noise at the local density (MODE 4, Sec. IV and Sec. V B): the draws of normals19;
@@ -154,29 +173,21 @@ __device__ __forceinline__ void normals19(const Step3Args<R>& a, uint32_t node, 
 // sqrt(rho)
 template <typename R>
 __device__ __forceinline__ void normals19_local(const Step3Args<R>& a, uint32_t node, R dr, R xi[Q3]) {
-    const uint4 ra = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, Lat19::TAG0), a.rk);
-    const uint4 rb = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, Lat19::TAG0 + 1), a.rk);
-    R n4, n16, spare;
-    lbf::gauss_word(ra.x, &n4, &xi[5]);
-    lbf::gauss_word(ra.y, &xi[6], &xi[7]);
-    lbf::gauss_word(ra.z, &xi[8], &xi[9]);
-    lbf::gauss_word(ra.w, &xi[10], &xi[11]);
-    lbf::gauss_word(rb.x, &xi[12], &xi[13]);
-    lbf::gauss_word(rb.y, &xi[14], &xi[15]);
-    lbf::gauss_word(rb.z, &n16, &xi[17]);
-    lbf::gauss_word(rb.w, &xi[18], &spare);
-    (void)spare;
+    const R G = sizeof(R) == 4 ? R(lbf::GAUSS_SCALE) : R(1);
+    R nu[16];
+    node_normals<Lat19::TAG0, 2>(a, node, nu);
     const R rho = a.co.rho0 + dr;
     const R c = a.cq[0] + dr * (a.cq[1] + dr * (a.cq[2] + dr * a.cq[3]));
     const R sr = lbf::sqrt_fast(fmax(rho, R(0)));
 #pragma unroll
-    for (int q = 5; q < Q3; ++q) xi[q] *= sr * a.sc[q];
+    for (int q = 5; q < Q3; ++q) xi[q] = nu[q - 4] * (sr * a.sc[q]);
     const R y44 = rho * (a.Lc[0] + a.Lb[0] * c);
     const R y416 = rho * (a.Lc[1] + a.Lb[1] * c);
     const R y1616 = rho * (a.Lc[2] + a.Lb[2] * c);
     const R L44 = lbf::sqrt_fast(fmax(y44, R(0)));
     const R L164 = L44 > R(0) ? y416 * lbf::recip(L44) : R(0);
     const R L1616 = lbf::sqrt_fast(fmax(y1616 - L164 * L164, R(0)));
+    const R n4 = G * nu[0], n16 = G * nu[12];
     xi[4] = L44 * n4;
     xi[16] = L164 * n4 + L1616 * n16;
 }
@@ -188,14 +199,7 @@ __host__ __device__ constexpr int nc27(int k) { return k - (k > 0) - (k > 1) - (
 template <typename R>
 __device__ __forceinline__ void normals27(const Step3Args<R>& a, uint32_t node, R xi[Q27]) {
     R nu[24];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const uint4 r = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, Lat27::TAG0 + d), a.rk);
-        lbf::gauss_word(r.x, &nu[8 * d + 0], &nu[8 * d + 1]);
-        lbf::gauss_word(r.y, &nu[8 * d + 2], &nu[8 * d + 3]);
-        lbf::gauss_word(r.z, &nu[8 * d + 4], &nu[8 * d + 5]);
-        lbf::gauss_word(r.w, &nu[8 * d + 6], &nu[8 * d + 7]);
-    }
+    node_normals<Lat27::TAG0, 3>(a, node, nu);
 #pragma unroll
     for (int k = 0; k < Q27; ++k)
         xi[k] = (k == 0 || k == 1 || k == 3 || k == 9) ? R(0) : a.sc[k] * nu[nc27(k)];
@@ -214,14 +218,7 @@ __device__ __forceinline__ void normals27(const Step3Args<R>& a, uint32_t node, 
 template <typename R>
 __device__ __forceinline__ void normals27_local(const Step3Args<R>& a, uint32_t node, R dr, R xi[Q27]) {
     R nu[24];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const uint4 r = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, Lat27::TAG0 + d), a.rk);
-        lbf::gauss_word(r.x, &nu[8 * d + 0], &nu[8 * d + 1]);
-        lbf::gauss_word(r.y, &nu[8 * d + 2], &nu[8 * d + 3]);
-        lbf::gauss_word(r.z, &nu[8 * d + 4], &nu[8 * d + 5]);
-        lbf::gauss_word(r.w, &nu[8 * d + 6], &nu[8 * d + 7]);
-    }
+    node_normals<Lat27::TAG0, 3>(a, node, nu);
     const R rho = a.co.rho0 + dr;
     const R c = a.cq[0] + dr * (a.cq[1] + dr * (a.cq[2] + dr * a.cq[3]));
     const R sr = lbf::sqrt_fast(fmax(rho, R(0)));
@@ -249,7 +246,10 @@ __device__ __forceinline__ void normals27_local(const Step3Args<R>& a, uint32_t 
     for (int r = 0; r < 7; ++r) {
         R s = R(0);
 #pragma unroll
-        for (int q = 0; q <= r; ++q) s += L[r * (r + 1) / 2 + q] * nu[nc27(coupled27(q))];
+        for (int q = 0; q <= r; ++q)
+            s += L[r * (r + 1) / 2 + q] *
+                 (sizeof(R) == 4 ? nu[nc27(coupled27(q))] * R(lbf::GAUSS_SCALE * sign27(coupled27(q)))
+                                 : nu[nc27(coupled27(q))]);
         xi[coupled27(r)] = s;
     }
 }
@@ -274,6 +274,8 @@ template <typename LAT, typename R>
 __device__ __forceinline__ R drho_of(const R* f) {
     if constexpr (LAT::Q == 19) {
         return drho19(f);
+    } else if constexpr (sizeof(R) == 4) {
+        return drho27_pairs(f);
     } else {
         R s = f[0];
 #pragma unroll
@@ -359,15 +361,28 @@ struct Slot3 {
     __host__ __device__ static constexpr int col(int cx) { return TMA ? XO - 1 - cx : 0; }
 };
 
+// density slots: planes z-1, z, z+1 and, with TMA, one more, so that the densities of plane z+1 are not
+// written where a slower warp still reads those of plane z-2
+template <bool TMA>
+__host__ __device__ constexpr int density_slots() { return TMA ? 4 : 3; }
+
+// Whether a plane has a barrier after its TMA wait as well.  With correlated noise it must: the box
+// contributions of the last plane are read until then.  Elsewhere the fourth density slot makes the wait
+// on the mbarrier enough, which is faster without noise (D3Q19 256^3: 582 -> 540 us); but under the
+// uncorrelated noise's arithmetic the four D3Q19 CTAs of an SM gain from the warps of a CTA staying
+// together (621 us with one barrier, 599 with two).
+template <typename LAT, int MODE>
+__host__ __device__ constexpr bool two_barriers() { return MODE == 3 || (LAT::Q == 19 && MODE == 1); }
+
 // Shared memory of the staged kernel: [SLOTS][SLOT] raw values, the mbarriers (TMA), the
-// density ring [3][RN], and with correlated noise (MODE 3) the 2x2x2-box contributions: for
+// density ring [3 or 4][RN], and with correlated noise (MODE 3) the 2x2x2-box contributions: for
 // the tile plus its left column and bottom row, the in-plane half (four pairs) of the current
 // plane and the upward half of the current and the previous plane.
 template <typename LAT, typename R, int TY, int SLOTS, int MODE, bool TMA>
 constexpr int staged_smem_bytes() {
     using S = Slot3<LAT, R, TY, TMA>;
     constexpr int HV = MODE == 3 ? 12 * RS_NV * (LAT::TX + 1) * (TY + 1) : 0;
-    return (SLOTS * S::SLOT + 3 * S::RN + HV) * (int)sizeof(R) + (TMA ? 16 * ((SLOTS + 1) / 2) : 0);
+    return (SLOTS * S::SLOT + density_slots<TMA>() * S::RN + HV) * (int)sizeof(R) + (TMA ? 16 * ((SLOTS + 1) / 2) : 0);
 }
 
 // resident CTAs per SM the register budget is sized for: as many as the shared memory admits
@@ -383,15 +398,17 @@ template <typename LAT, typename R, int TY, int MODE, typename I, int SLOTS, boo
 __global__ void __launch_bounds__(LAT::TX * TY, staged_min_blocks<LAT, R, TY, SLOTS, MODE, TMA>())
     step3_staged_kernel(const __grid_constant__ CUtensorMap tmap, const Step3Args<R> a) {
     constexpr int Q = LAT::Q, TX = LAT::TX;
+    constexpr bool TWO = two_barriers<LAT, MODE>();
     using S = Slot3<LAT, R, TY, TMA>;
     constexpr int RX = S::RX, RN = S::RN, NT = TX * TY, SL = S::SLOT, BW = S::BW;
     extern __shared__ __align__(128) unsigned char smem3[];
     R* raw = reinterpret_cast<R*>(smem3);                                   // [SLOTS][SL]
     constexpr int RAW_BYTES = SLOTS * SL * (int)sizeof(R);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem3 + RAW_BYTES);         // TMA: one per slot
-    R* rs = reinterpret_cast<R*>(smem3 + RAW_BYTES + (TMA ? 16 * ((SLOTS + 1) / 2) : 0));   // [3][RN]
+    constexpr int ND = density_slots<TMA>();
+    R* rs = reinterpret_cast<R*>(smem3 + RAW_BYTES + (TMA ? 16 * ((SLOTS + 1) / 2) : 0));   // [ND][RN]
     constexpr int HW = TX + 1, HN = HW * (TY + 1), NV = RS_NV;
-    R* Hin = rs + 3 * RN;                                   // MODE 3: [4][NV][HN] in-plane half
+    R* Hin = rs + ND * RN;                                  // MODE 3: [4][NV][HN] in-plane half
     R* Hup = Hin + 4 * NV * HN;                             // MODE 3: [2][4][NV][HN] upward half
     const int nx = a.nx, ny = a.ny, nz = a.nz, pitch = a.pitch, GX = a.gx;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
@@ -411,6 +428,8 @@ __global__ void __launch_bounds__(LAT::TX * TY, staged_min_blocks<LAT, R, TY, SL
         }
         __syncthreads();
     }
+    lbf::grid_wait();
+    lbf::grid_next();
 
     // Copies: the ring positions a thread stages are the same on every plane; their stored
     // in-plane offsets (no wrap: the ghosts cover the ring) and validity are formed once.
@@ -463,21 +482,29 @@ __global__ void __launch_bounds__(LAT::TX * TY, staged_min_blocks<LAT, R, TY, SL
             cp_async_commit();
         }
     };
-    // wait until raw slot k has landed and is visible to the whole CTA (a block-wide barrier
-    // either way); false, for every thread, if any thread gave up on a TMA wait
+    // wait until raw slot k has landed.  TMA: every thread waits on the slot's mbarrier, which makes the
+    // values visible to it; false if it gave up, which the plane's barrier makes known to all (what
+    // such a thread reads meanwhile goes nowhere).  Copies: a block-wide barrier.
     auto wait_slot = [&](int slot_k) -> bool {
         if constexpr (TMA) {
             const uint32_t par = (phase >> slot_k) & 1u;
             const bool ok = lbf::mbar_wait_bounded(lbf::smem_u32(&bar[slot_k]), par);
-            if (__syncthreads_or(!ok)) return false;
-            phase ^= 1u << slot_k;
-            pending &= ~(1u << slot_k);
-            return true;
+            if (ok) {
+                phase ^= 1u << slot_k;
+                pending &= ~(1u << slot_k);
+            }
+            return ok;
         } else {
             cp_async_wait_all();
             __syncthreads();
             return true;
         }
+    };
+    // the plane's barrier; false, for every thread, if any gave up on a TMA wait
+    auto plane_barrier = [&](bool ok) -> bool {
+        if constexpr (TMA) return !__syncthreads_or(!ok);
+        __syncthreads();
+        return true;
     };
     // a CTA that gave up sets the error word and gives its loads in flight a bounded chance
     // to land in its shared memory before it exits
@@ -538,33 +565,62 @@ __global__ void __launch_bounds__(LAT::TX * TY, staged_min_blocks<LAT, R, TY, SL
             const uint4 r1 = lbf::philox4x32_10(make_uint4(node, a.t_lo, a.t_hi, rs_tag<LAT>() + 1), a.rk);
             const uint32_t wd[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
             R vx[8], vy[8];
+            if constexpr (sizeof(R) == 4) {
+                // words two at a time; the transform's levels 2 and 4 on pairs of words, level 1 within
+                F2 px[4], py[4];
 #pragma unroll
-            for (int w = 0; w < 8; ++w) {
-                R n0, n1;
-                lbf::gauss_word(wd[w], &n0, &n1);
-                const int cls = rs_class<LAT>((w & 1) + ((w >> 1) & 1) + ((w >> 2) & 1));
-                vx[w] = a.Lrs[3 * cls] * n0;
-                if constexpr (LAT::Q == 19)
-                    vy[w] = a.Lrs[3 * cls + 1] * n0 + a.Lrs[3 * cls + 2] * n1;
-                else
-                    vy[w] = a.Lrs[3 * cls + 2] * n1;
-            }
+                for (int k = 0; k < 4; ++k) {
+                    auto cls = [](int w) { return rs_class<LAT>((w & 1) + ((w >> 1) & 1) + ((w >> 2) & 1)); };
+                    const int c0 = 3 * cls(2 * k), c1 = 3 * cls(2 * k + 1);
+                    F2 n0, n1;
+                    lbf::gauss2(wd[2 * k], wd[2 * k + 1], &n0, &n1);
+                    px[k] = mul2(n0, make_float2(a.Lrs[c0], a.Lrs[c1]));
+                    py[k] = mul2(n1, make_float2(a.Lrs[c0 + 2], a.Lrs[c1 + 2]));
+                    if constexpr (LAT::Q == 19)
+                        py[k] = fma2(n0, make_float2(a.Lrs[c0 + 1], a.Lrs[c1 + 1]), py[k]);
+                }
+                auto wht = [](const F2 (&p)[4], R* v) {
+                    const F2 s0 = add2(p[0], p[1]), d0 = sub2(p[0], p[1]), s1 = add2(p[2], p[3]), d1 = sub2(p[2], p[3]);
+                    const F2 q[4] = {add2(s0, s1), add2(d0, d1), sub2(s0, s1), sub2(d0, d1)};
 #pragma unroll
-            for (int b = 1; b < 8; b <<= 1)
-#pragma unroll
-                for (int w = 0; w < 8; ++w)
-                    if (!(w & b)) {
-                        const R ax = vx[w], ay = vy[w], bx = vx[w | b], by = vy[w | b];
-                        vx[w] = ax + bx; vy[w] = ay + by;
-                        vx[w | b] = ax - bx; vy[w | b] = ay - by;
+                    for (int k = 0; k < 4; ++k) {
+                        const F2 t = sum_diff(q[k].x, q[k].y);
+                        v[2 * k] = t.x;
+                        v[2 * k + 1] = t.y;
                     }
+                };
+                wht(px, vx);
+                wht(py, vy);
+            } else {
+#pragma unroll
+                for (int w = 0; w < 8; ++w) {
+                    R n0, n1;
+                    lbf::gauss_word(wd[w], &n0, &n1);
+                    const int cls = rs_class<LAT>((w & 1) + ((w >> 1) & 1) + ((w >> 2) & 1));
+                    vx[w] = a.Lrs[3 * cls] * n0;
+                    if constexpr (LAT::Q == 19)
+                        vy[w] = a.Lrs[3 * cls + 1] * n0 + a.Lrs[3 * cls + 2] * n1;
+                    else
+                        vy[w] = a.Lrs[3 * cls + 2] * n1;
+                }
+#pragma unroll
+                for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+                    for (int w = 0; w < 8; ++w)
+                        if (!(w & b)) {
+                            const R ax = vx[w], ay = vy[w], bx = vx[w | b], by = vy[w | b];
+                            vx[w] = ax + bx; vy[w] = ay + by;
+                            vx[w | b] = ax - bx; vy[w | b] = ay - by;
+                        }
+            }
+            const R unit = sizeof(R) == 4 ? R(1) : R(0.125);       // FP32: in Lrs
 #pragma unroll
             for (int m = 0; m < 8; ++m) {
                 R* dst = (m & 1) ? Hup + ub * 4 * NV * HN : Hin;
                 if (!(m & 1) && !keep_in) continue;
                 const int j = m >> 1;
-                dst[(j * NV) * HN + p] = R(0.125) * vx[m];
-                dst[(j * NV + 1) * HN + p] = R(0.125) * vy[m];
+                dst[(j * NV) * HN + p] = unit * vx[m];
+                dst[(j * NV + 1) * HN + p] = unit * vy[m];
             }
         }
     };
@@ -608,7 +664,8 @@ __global__ void __launch_bounds__(LAT::TX * TY, staged_min_blocks<LAT, R, TY, SL
                 xi[4] = s4;
                 xi[16] = s16;
             }
-            collide19(a.co, f, r, xi, o);
+            if constexpr (sizeof(R) == 4 && MODE == 3) collide19_f(a.co, a.lam, f, r, xi, o);
+            else collide19(a.co, f, r, xi, o);
         } else {
             // nb[i] = rho(r + c_i)
             R nb[Q27];
@@ -635,35 +692,43 @@ __global__ void __launch_bounds__(LAT::TX * TY, staged_min_blocks<LAT, R, TY, SL
 #pragma unroll
                 for (int r = 0; r < 7; ++r) xi[coupled27(r)] += a.Prs[r] * sp + a.Qrs[r] * sq;
             }
-            collide27(a.co, f, nb, xi, o);
+            if constexpr (sizeof(R) == 4) collide27_f<MODE != 0>(a.co, f, nb, xi, o);
+            else collide27(a.co, f, nb, xi, o);
         }
         store_node3<LAT, R, I>(a, (I)z * PLI, x, y, o);
     };
 
     if constexpr (SLOTS == 3) {
-        // planes z0-1, z0 -> slots 0, 1; plane z0+1 -> slot 2 (in flight); density slots alike
+        // planes z0-1, z0 -> raw slots 0, 1; plane z0+1 -> slot 2 (in flight); density slots alike
         issue(z0 - 1, 0);
         issue(z0, 1);
         if constexpr (TMA) issue(z0 + 1, 2);
-        if (!wait_slot(0) || !wait_slot(1)) { give_up(); return; }
+        bool ok = wait_slot(0);
+        ok = wait_slot(1) && ok;
         density(0, 0);
         density(1, 1);
         if constexpr (MODE == 3) stencil_plane(z0 - 1, false, 0);
         if constexpr (!TMA) issue(z0 + 1, 2);
+        else if (!plane_barrier(ok)) { give_up(); return; }
         for (int z = z0; z < z1; ++z) {
-            const int k0 = (z - z0 + 1) % 3, km = (k0 + 2) % 3, kp = (k0 + 1) % 3;   // slots of z, z-1, z+1
-            if (!wait_slot(kp)) { give_up(); return; }
-            if (TMA && z + 1 < z1) issue(z + 2, km);    // plane z-1's slot is free
-            density(kp, kp);
+            const int r0 = (z - z0 + 1) % 3, rm = (r0 + 2) % 3, rp = (r0 + 1) % 3;    // raw slots of z, z-1, z+1
+            const int k0 = (z - z0 + 1) % ND, km = (k0 + ND - 1) % ND, kp = (k0 + 1) % ND;   // density slots
+            ok = wait_slot(rp);
+            if constexpr (TMA && TWO) {
+                if (!plane_barrier(ok)) { give_up(); return; }
+            }
+            density(rp, kp);
             if constexpr (MODE == 3) stencil_plane(z, true, (z - z0 + 1) & 1);
-            if (!TMA && z + 1 < z1) issue(z + 2, km);
-            __syncthreads();
-            if (!own) continue;
-            const R* sl = raw + k0 * SL;
-            R f[Q];
+            if (!TMA && z + 1 < z1) issue(z + 2, rm);
+            if (!plane_barrier(ok)) { give_up(); return; }
+            if (own) {
+                const R* sl = raw + r0 * SL;
+                R f[Q];
 #pragma unroll
-            for (int i = 0; i < Q; ++i) f[i] = sl[S::pbase(i) + qb + S::col(LAT::c(i, 0))];
-            collide_plane(z, f, k0, km, kp, (z - z0) & 1);
+                for (int i = 0; i < Q; ++i) f[i] = sl[S::pbase(i) + qb + S::col(LAT::c(i, 0))];
+                if (TMA && z + 1 < z1) issue(z + 2, rm);     // plane z-1's slot is free
+                collide_plane(z, f, k0, km, kp, (z - z0) & 1);
+            }
         }
     } else {
         // two raw slots: a plane's own pulled values move to registers when its densities are
@@ -676,22 +741,29 @@ __global__ void __launch_bounds__(LAT::TX * TY, staged_min_blocks<LAT, R, TY, SL
         };
         issue(z0 - 1, 0);
         issue(z0, 1);
-        if (!wait_slot(0) || !wait_slot(1)) { give_up(); return; }
+        bool ok = wait_slot(0);
+        ok = wait_slot(1) && ok;
         density(0, 0);                 // plane z0-1 -> density slot 0
         density(1, 1);                 // plane z0 -> density slot 1
         take(1, fcur);
         if constexpr (MODE == 3) stencil_plane(z0 - 1, false, 0);
-        __syncthreads();
+        if (!plane_barrier(ok)) { give_up(); return; }
         issue(z0 + 1, 0);              // raw slot of plane p: (p - z0 + 1) % 2
         for (int z = z0; z < z1; ++z) {
-            const int k0 = (z - z0 + 1) % 3, km = (k0 + 2) % 3, kp = (k0 + 1) % 3;
+            const int k0 = (z - z0 + 1) % ND, km = (k0 + ND - 1) % ND, kp = (k0 + 1) % ND;   // density slots of z, z-1, z+1
             const int rp = (z - z0) & 1;             // raw slot of plane z+1
-            if (!wait_slot(rp)) { give_up(); return; }
-            if (z + 1 < z1) issue(z + 2, rp ^ 1);    // the slot of plane z, already in registers
+            // the slot of plane z, in registers since before the last barrier (TMA; by copies, whose
+            // threads share a slot's loads, after the wait)
+            if (TMA && !TWO && z + 1 < z1) issue(z + 2, rp ^ 1);
+            ok = wait_slot(rp);
+            if constexpr (TMA && TWO) {
+                if (!plane_barrier(ok)) { give_up(); return; }
+            }
+            if ((!TMA || TWO) && z + 1 < z1) issue(z + 2, rp ^ 1);
             density(rp, kp);
             take(rp, fnext);
             if constexpr (MODE == 3) stencil_plane(z, true, (z - z0 + 1) & 1);
-            __syncthreads();
+            if (!plane_barrier(ok)) { give_up(); return; }
             if (own) collide_plane(z, fcur, k0, km, kp, (z - z0) & 1);
 #pragma unroll
             for (int i = 0; i < Q; ++i) fcur[i] = fnext[i];
@@ -740,7 +812,7 @@ __global__ void __launch_bounds__(TX * TY) step3_kernel(const Step3Args<R> a) {
             if (gx <= nx && gy <= ny) {
                 R f[Q3];
                 pull19(src, P, Zs, (long long)(gy + GY3) * pitch + gx + GX, pitch, f);
-                v = drho19(f);
+                v = drho_of<Lat19>(f);
             }
             rs[slot][ly][lx] = v;
         }
@@ -819,8 +891,7 @@ static cudaError_t launch_staged(const Step3Args<R>& a, const CUtensorMap* map, 
             if (e != cudaSuccess) return e;
             done.fetch_or(bit, std::memory_order_release);
         }
-        kern<<<grid, LAT::TX * TY, smem, s>>>(*map, a);
-        return cudaGetLastError();
+        return lbf::launch_chained(kern, grid, dim3(LAT::TX * TY), smem, s, *map, a);
     }
 }
 
