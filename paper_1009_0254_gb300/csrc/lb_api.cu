@@ -773,16 +773,18 @@ int lb_set_populations(lb_ctx* c, const double* f, int loc, int64_t t) {
 int lb_get_populations(lb_ctx* c, double* f, int loc) {
     if (!c || !f || (loc != LB_HOST && loc != LB_DEVICE)) return LB_EINVAL;
     DeviceGuard dg(c->device);
+    if (loc == LB_DEVICE) {
+        CK(c, launch_get_all(c->pop[c->cur], c->precision, c->g, c->fbar, f, c->stream), "get populations");
+        c->kernels += 1;
+        return check_device_error(c);          // synchronises
+    }
     double* stage = (double*)c->z1;
     for (int i = 0; i < Q; ++i) {
-        double* dst = (loc == LB_HOST) ? stage : f + (long long)i * c->n;
-        CK(c, launch_get_plane(c->pop[c->cur], c->precision, c->g, i, c->fbar[i], dst, c->stream), "get populations");
+        CK(c, launch_get_plane(c->pop[c->cur], c->precision, c->g, i, c->fbar[i], stage, c->stream), "get populations");
         c->kernels += 1;
-        if (loc == LB_HOST)
-            CK(c, cudaMemcpyAsync(f + (long long)i * c->n, stage, sizeof(double) * c->n, cudaMemcpyDeviceToHost,
-                                  c->stream), "D2H");
+        CK(c, cudaMemcpyAsync(f + (long long)i * c->n, stage, sizeof(double) * c->n, cudaMemcpyDeviceToHost, c->stream),
+           "D2H");
     }
-    CK(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
     return check_device_error(c);
 }
 

@@ -1086,16 +1086,19 @@ int lb_batch_get_populations(lb_batch* b, int replica, double* f, int loc) {
     const long long n = (long long)ci.nx * ci.ny;
     double* stage = reinterpret_cast<double*>(cls_ptr(b, b->L.off_stage));
     const void* pops = rep_pops(b, replica, (int)(b->K & 1));
-    for (int i = 0; i < Q; ++i) {
-        double* dst = loc == LB_HOST ? stage : f + i * n;
-        BCK(b, launch_get_plane(pops, 0, ci.g, i, b->fbar[i], dst, b->stream), "get populations");
+    if (loc == LB_DEVICE) {
+        BCK(b, launch_get_all(pops, 0, ci.g, b->fbar, f, b->stream), "get populations");
         b->kernels++;
-        if (loc == LB_HOST)
+    } else {
+        for (int i = 0; i < Q; ++i) {
+            BCK(b, launch_get_plane(pops, 0, ci.g, i, b->fbar[i], stage, b->stream), "get populations");
+            b->kernels++;
             BCK(b, cudaMemcpyAsync(f + i * n, stage, sizeof(double) * n, cudaMemcpyDeviceToHost, b->stream), "D2H");
+        }
     }
-    BCK(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
     int h = 0;
-    BCK(b, cudaMemcpy(&h, cls_ptr(b, b->L.off_err), sizeof(int), cudaMemcpyDeviceToHost), "D2H");
+    BCK(b, cudaMemcpyAsync(&h, cls_ptr(b, b->L.off_err), sizeof(int), cudaMemcpyDeviceToHost, b->stream), "D2H");
+    BCK(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
     if (h) return bfail(b, LB_ETIMEOUT, "a batched step kernel gave up waiting for its TMA loads");
     return LB_OK;
 }

@@ -70,6 +70,17 @@ struct Elem<double> {
     __host__ __device__ static __forceinline__ double store(double v, int) { return v; }
 };
 
+// (double)x by moving the fields of x: a conversion takes the FP64 pipe, two a clock and SM, and with the
+// addition of the rest value made the read-back of a state FP64 bound.  The exponent's bias grows by 896
+// (subnormals are normalised first; infinities and NaN keep an exponent of ones).
+__device__ __forceinline__ double widen(float x) {
+    const bool small = fabsf(x) < 1.17549435e-38f;
+    const uint32_t b = __float_as_uint(small ? x * 16777216.0f : x), mag = b & 0x7fffffffu;
+    const uint32_t add = small ? (mag ? 872u << 20 : 0u) : (mag >= 0x7f800000u ? 1792u << 20 : 896u << 20);
+    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + add)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // arithmetic type of a storage type, and its complex pair
 template <typename T>
 struct Arith {
@@ -469,6 +480,9 @@ cudaError_t launch_set_plane(const double* src, void* pops, int storage, const G
                              cudaStream_t s);
 cudaError_t launch_get_plane(const void* pops, int storage, const Grid& g, int i, double fbar, double* out,
                              cudaStream_t s);
+// every population to FP64 at once, out[i][y][x]
+cudaError_t launch_get_all(const void* pops, int storage, const Grid& g, const double fbar[Q], double* out,
+                           cudaStream_t s);
 cudaError_t launch_moment(const void* pops, int storage, const Grid& g, int a, const double* fbar9, double* out,
                           cudaStream_t s);
 cudaError_t launch_sums(const void* pops, int storage, const Grid& g, const double* fbar9, double* partial,
