@@ -211,6 +211,7 @@ struct lb_ctx {
     unsigned short* bin16 = nullptr;     // radial bin of every wavevector (spectra)
     int* err_dev = nullptr;          // set by a kernel whose bounded wait gave up
     bool pow2 = false;
+    bool use_resident = false;      // small lattices: many steps a launch, state in shared memory
     bool use_tma = false;            // TMA-staged persistent step kernel
     bool use_sweep = false;          // warp-autonomous vertical sweep kernel
     int sweep_occ6 = 0;              // its occupancy variant
@@ -369,8 +370,9 @@ int lb_create(int nx, int ny, int precision, uint64_t seed, double rho0, double 
     c->err_dev = (int*)(c->ws + c->L.err);
     rest_populations(rho0, cs2, c->fbar);
     {
-        // LBFLUCT_STEP_KERNEL=simple selects the plain kernel; LBFLUCT_TMA_TILE=<0..4> fixes a
-        // tile shape (otherwise each step uses the fastest one for its noise mode)
+        // LBFLUCT_STEP_KERNEL=tma selects the TMA-staged kernel for lattices of every size, =simple the
+        // plain kernel; LBFLUCT_TMA_TILE=<0..4> fixes the former's tile shape (otherwise each step uses
+        // the fastest one for its noise mode)
         const char* v = std::getenv("LBFLUCT_STEP_KERNEL");
         c->use_sweep = v && (std::strcmp(v, "sweep") == 0 || std::strcmp(v, "sweep6") == 0) && sweep_fits(g);
         c->sweep_occ6 = v && std::strcmp(v, "sweep6") == 0;
@@ -378,6 +380,7 @@ int lb_create(int nx, int ny, int precision, uint64_t seed, double rho0, double 
         // FP64 storage runs the plain kernel (its arithmetic is FP64 throughout)
         const bool want_tma = !(v && std::strcmp(v, "simple") == 0) && !c->use_sweep && precision != LB_FP64;
         const char* tv = std::getenv("LBFLUCT_TMA_TILE");
+        c->use_resident = !v && !tv && precision != LB_FP64 && resident_fits(g) && resident_available();
         c->tma_tile_fixed = tv ? std::atoi(tv) : -1;
         if (c->tma_tile_fixed >= tma_tile_count()) c->tma_tile_fixed = -1;
         c->tma_tile = c->tma_tile_fixed >= 0 ? c->tma_tile_fixed : tma_default_tile(LB_NOISE_LW, c->fp16);
@@ -652,7 +655,35 @@ int lb_step(lb_ctx* c, int64_t nsteps) {
                          : (c->noise_mode == LB_NOISE_FULL_RS ? 3 : (c->noise_mode == LB_NOISE_LW_LOCAL ? 4 : 1)));
     if (kmode == 2 && !c->pow2)
         return fail(c, LB_EINVAL, "correlated noise needs nx and ny powers of two (radix-2 FFT)");
+    // Small lattices: as many steps a launch as there are to the end or the next sample (4,096 at most, so
+    // that a launch stays within some milliseconds).  A launch costs 5.5 us, a step 1.0 to 2.7 us in it and
+    // 3.7 by itself: two steps of 64^2 took 4.1 us a step against 3.8, four 2.6; four of 128^2 4.1 against
+    // 3.8, eight 3.3.  Hence four steps, and eight above 8,192 nodes.  Kernel timing asks for a launch per
+    // step; the FP16 double well is the plain kernel's.
+    const bool poly2 = c->eos == LB_EOS_DOUBLE_WELL;
+    const bool resident = c->use_resident && c->timing == 0 && (kmode < 2 || kmode == 4) && !(poly2 && c->fp16);
     for (int64_t k = 0; k < nsteps; ++k) {
+        if (resident) {
+            int64_t m = std::min<int64_t>(nsteps - k, 4096);
+            if (c->every > 0) m = std::min<int64_t>(m, c->every - c->t % c->every);
+            if (m >= (c->n <= 8192 ? 4 : 8)) {
+                StepArgs a = c->sa;
+                a.src = c->pop[c->cur];
+                a.dst = c->pop[c->cur ^ 1];
+                CK(c, launch_step_resident(a, c->sad, c->t, (int)m, kmode, c->fp16, poly2, c->stream), "step kernel launch");
+                c->kernels += 1;
+                c->cur ^= 1;
+                c->t += m;
+                k += m - 1;
+                if (c->every > 0 && c->t % c->every == 0) {
+                    CK(c, launch_stats_sample(c->pop[c->cur], c->precision, c->g, c->z1, c->z2, c->twx, c->twy, c->bin16,
+                                              c->bins, c->nbins, c->stream), "spectra sample");
+                    c->kernels += 6;
+                    c->nsamples++;
+                }
+                continue;
+            }
+        }
         const uint32_t tlo = (uint32_t)((uint64_t)c->t & 0xffffffffu), thi = (uint32_t)((uint64_t)c->t >> 32);
         if (c->precision == LB_FP64) {
             // FP64 storage: FP64 noise synthesis and the plain kernel in FP64

@@ -463,6 +463,11 @@ bool make_pop_tensor_maps(const void* buf, const Grid& g, int tile, int fp16, vo
 int tma_tile_count();
 int tma_default_tile(int noise_mode, int fp16);
 size_t tensor_map_bytes();
+// many steps of a small lattice in one launch (lb_step_resident.cu)
+bool resident_fits(const Grid& g);
+bool resident_available();
+cudaError_t launch_step_resident(const StepArgs& a, const StepArgsD& d, long long t, int nsteps, int noise_mode, int fp16,
+                                 bool poly, cudaStream_t s);
 cudaError_t launch_noise49(float2* buf, float2* scratch, const NoiseGenArgs& ga, const float2* twx,
                            const float2* twy, cudaStream_t s);
 cudaError_t launch_noise49_d(double2* buf, const NoiseGenArgsD& ga, const double2* twx, const double2* twy,
