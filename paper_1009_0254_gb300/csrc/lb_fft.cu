@@ -298,8 +298,12 @@ cudaError_t launch_stats_sample(const void* pops, int storage, const Grid& g, fl
     e = cudaFuncSetAttribute(bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const long long units = (long long)(g.ny / 2 + 1) * ((g.nx / 2 + 32) / 32);   // warp work units
-    const int nblk = (int)std::min<long long>(304, std::max<long long>(1, units / 32));   // <= 2 per SM
-    bin_kernel<<<nblk, 256, smem, s>>>(z1, z2, bin16, g.nx, g.ny, nbins, bins);
+    // two CTAs per SM, of 16 warps where there are four units for each (a warp's loads of a unit are one
+    // latency: 4096^2 a sample 619 us with 8 warps, 554 with 16; 2048^2 155, 144), of 8 below (256^2 37.6
+    // against 38.5; four CTAs per SM of 8 warps lose at 4,096 bins, 98 KB each: 636)
+    const int threads = units >= 304 * 64 ? 512 : 256;
+    const int nblk = (int)std::min<long long>(304, std::max<long long>(1, units * 8 / threads));
+    bin_kernel<<<nblk, threads, smem, s>>>(z1, z2, bin16, g.nx, g.ny, nbins, bins);
     return cudaGetLastError();
 }
 
