@@ -28,7 +28,7 @@
 // Step at 4096^2, before and after this form (scalar nodes, two stages, stores by thread):
 // FP32 without noise 262 -> 186 us, uncorrelated 212 -> 191 (6.32 TB/s of the 72 bytes a node),
 // k-space correlated (the step kernel) 235 -> 221 less launch, real space 333 -> 263, local
-// density 219 -> 194; FP16 uncorrelated 220 -> 182, 209 instructions a node against 341.  What
+// density 219 -> 194; FP16 uncorrelated 220 -> 182, 237 instructions a node against 375.  What
 // bounds it now: FP32 DRAM; FP16 and the real-space noise the SM (FMA-heavy pipe 60 % busy, half
 // of it the wide multiplies of Philox, and the barriers between the passes).
 //
