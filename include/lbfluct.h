@@ -48,7 +48,9 @@ extern "C" {
 #define LB_FP32 0          /* FP32 deviations f_i - fbar_i (72 bytes moved per node update) */
 #define LB_FP16DEV 1       /* FP16 deviations, stored as (f_i - fbar_i) / w_i (36 bytes per node update);
                               arithmetic stays FP32; rounding to FP16 each step makes the mass
-                              conserved only to that rounding */
+                              conserved only to that rounding.  The state and its sampled spectra
+                              repeat from run to run; with sums taken in another order (another
+                              step kernel) they are equal to FP16 rounding, 2^-11 of a value, only */
 #define LB_FP64 2          /* FP64 deviations and FP64 arithmetic throughout the step (the
                               correlated noise too, which then needs ny <= 4096); the sampled
                               spectra are FP32 transforms accumulated in FP64 */

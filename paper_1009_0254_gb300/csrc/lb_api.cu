@@ -380,7 +380,7 @@ int lb_create(int nx, int ny, int precision, uint64_t seed, double rho0, double 
         // FP64 storage runs the plain kernel (its arithmetic is FP64 throughout)
         const bool want_tma = !(v && std::strcmp(v, "simple") == 0) && !c->use_sweep && precision != LB_FP64;
         const char* tv = std::getenv("LBFLUCT_TMA_TILE");
-        c->use_resident = !v && !tv && precision != LB_FP64 && resident_fits(g) && resident_available();
+        c->use_resident = !v && !tv && precision == LB_FP32 && resident_fits(g) && resident_available();
         c->tma_tile_fixed = tv ? std::atoi(tv) : -1;
         if (c->tma_tile_fixed >= tma_tile_count()) c->tma_tile_fixed = -1;
         c->tma_tile = c->tma_tile_fixed >= 0 ? c->tma_tile_fixed : tma_default_tile(LB_NOISE_LW, c->fp16);
@@ -659,9 +659,9 @@ int lb_step(lb_ctx* c, int64_t nsteps) {
     // that a launch stays within some milliseconds).  A launch costs 5.5 us, a step 1.0 to 2.7 us in it and
     // 3.7 by itself: two steps of 64^2 took 4.1 us a step against 3.8, four 2.6; four of 128^2 4.1 against
     // 3.8, eight 3.3.  Hence four steps, and eight above 8,192 nodes.  Kernel timing asks for a launch per
-    // step; the FP16 double well is the plain kernel's.
+    // step.
     const bool poly2 = c->eos == LB_EOS_DOUBLE_WELL;
-    const bool resident = c->use_resident && c->timing == 0 && (kmode < 2 || kmode == 4) && !(poly2 && c->fp16);
+    const bool resident = c->use_resident && c->timing == 0 && (kmode < 2 || kmode == 4);
     for (int64_t k = 0; k < nsteps; ++k) {
         if (resident) {
             int64_t m = std::min<int64_t>(nsteps - k, 4096);
@@ -670,7 +670,7 @@ int lb_step(lb_ctx* c, int64_t nsteps) {
                 StepArgs a = c->sa;
                 a.src = c->pop[c->cur];
                 a.dst = c->pop[c->cur ^ 1];
-                CK(c, launch_step_resident(a, c->sad, c->t, (int)m, kmode, c->fp16, poly2, c->stream), "step kernel launch");
+                CK(c, launch_step_resident(a, c->sad, c->t, (int)m, kmode, poly2, c->stream), "step kernel launch");
                 c->kernels += 1;
                 c->cur ^= 1;
                 c->t += m;
@@ -755,8 +755,9 @@ int lb_step(lb_ctx* c, int64_t nsteps) {
                     return fail(c, LB_ECUDA, "tensor map encoding failed");
                 c->tma_tile = want;
             }
-            CK(c, launch_step_tma(a, c->sad, c->tmap[c->cur], c->tmap_out[c->cur ^ 1], c->err_dev, kmode, c->tma_tile, c->fp16,
-                                  c->stream, poly),
+            CK(c, c->fp16 ? launch_step_half(a, c->tmap[c->cur], c->err_dev, kmode, c->tma_tile, c->stream)
+                          : launch_step_tma(a, c->sad, c->tmap[c->cur], c->tmap_out[c->cur ^ 1], c->err_dev, kmode,
+                                            c->tma_tile, c->stream, poly),
                "step kernel launch");
         } else
             CK(c, launch_step_simple(a, kmode, c->fp16, c->stream), "step kernel launch");

@@ -92,7 +92,7 @@ __device__ __forceinline__ TilePos locate(const EnsParams& p, int tile) {
 // raises the register count, so launches without such replicas use the lean variant)
 template <int TX, int TY, int NT, bool RS>
 __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_ensemble_kernel(const __grid_constant__ EnsParams p) {
-    using TT = TmaTile<TX, TY, float>;
+    using TT = TmaTile<TX, TY>;
     using M = PairMap<TX, TY, NT>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float* S = reinterpret_cast<float*>(smem_raw);
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
             tma_load_4d(smem_u32(S + i * TT::PS), map, tp.x0 - TT::XO + gx, tp.y0 - 1 - kCYt[i] + GY, i, tp.rep, bar);
     };
     auto store = [&](const TilePos& tp) {
-        if (tile_direct<TX, float>(p.cls[tp.c].g, tp.x0)) return;
+        if (tile_direct<TX>(p.cls[tp.c].g, tp.x0)) return;
         tma_store_4d(&p.out[tp.c][par ^ 1], smem_u32(out), tp.x0, tp.y0, 0, tp.rep);
         tma_store_commit();
     };
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
         // pulled populations stay in registers across the density barrier; the next tile is
         // loaded right after it
         F2 fr[M::RPT][Q], z4[M::RPT], z9[M::RPT];
-        tile_pull<TX, TY, NT, false, RS>(S, R, fr);
+        tile_pull<TX, TY, NT, RS>(S, R, fr);
         if (tid == 0) tma_store_wait_read();
         __syncthreads();
         if (tid == 0 && tn < ntiles) {
@@ -183,20 +183,20 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
             if (mode == 3) {
                 stencil_tile<TX, TY, NT>(sargs, xch, tp.x0, tp.y0, g.nx, g.ny, z4, z9);
                 __syncthreads();
-                tile_collide<3, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
+                tile_collide<3, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
                                                           z9, xch);
                 stepped = true;
             }
         }
         if (!stepped) {
             if (mode == 2)
-                tile_collide<2, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst,
+                tile_collide<2, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst,
                                                           d.xi + (long long)tp.rep * g.nx * g.ny, z4, z9, nullptr);
             else if (mode)
-                tile_collide<1, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
+                tile_collide<1, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
                                                           z9, nullptr);
             else
-                tile_collide<0, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
+                tile_collide<0, false, TX, TY, NT>(sargs, nullptr, fr, R, g, tp.x0, tp.y0, out, dst, nullptr, z4,
                                                           z9, nullptr);
         }
         fence_async_smem();
@@ -386,7 +386,7 @@ static bool make_class_maps(void* buf, const Grid& g, int R, int tile, CUtensorM
 // dynamic shared memory of the step kernel
 template <int TX, int TY, int NT, bool RS>
 constexpr int ensemble_smem() {
-    return TmaTile<TX, TY, float>::SMEM_BYTES + (RS ? StencilTile<TX, TY, NT>::BYTES : 0);
+    return TmaTile<TX, TY>::SMEM_BYTES + (RS ? StencilTile<TX, TY, NT>::BYTES : 0);
 }
 
 // CTAs of a persistent launch: every SM filled to the occupancy the kernel allows
@@ -441,7 +441,6 @@ static cudaError_t prepare_ensemble_kernels() {
 // offset are left to the caller.
 void fill_rep_record(double rho0, double cs2, double kT, double kappa, double tau_s, double tau_b,
                      double tau_ghost, int noise_mode, RepRec* rec) {
-    constexpr double c = pair_scale<false>();
     double xi[81];
     lb_noise_matrix(rho0, cs2, kT, kappa, tau_s, tau_b, tau_ghost, 0.0, 0.0, xi);
     const double x44 = xi[3 * 9 + 3], x49 = noise_mode == LB_NOISE_DIAG ? 0.0 : xi[3 * 9 + 8], x99 = xi[8 * 9 + 8];
@@ -451,7 +450,7 @@ void fill_rep_record(double rho0, double cs2, double kT, double kappa, double ta
     const double L[4] = {L44, 0.0, L94, L99};
     const double s3[3] = {std::sqrt(std::fmax(xi[4 * 9 + 4], 0.0)), std::sqrt(std::fmax(xi[5 * 9 + 5], 0.0)),
                           std::sqrt(std::fmax(xi[6 * 9 + 6], 0.0))};
-    pair_coef(rho0, cs2 - 1.0 / 3.0, kappa, -1.0 / tau_b, -1.0 / tau_s, -1.0 / tau_ghost, -1.0 / tau_ghost, L, s3, c,
+    pair_coef(rho0, cs2 - 1.0 / 3.0, kappa, -1.0 / tau_b, -1.0 / tau_s, -1.0 / tau_ghost, -1.0 / tau_ghost, L, s3,
               rec);
     double co[6];
     noise_coefficients(rho0, cs2, kT, kappa, tau_s, tau_b, tau_ghost, co);
@@ -469,7 +468,7 @@ void fill_rep_record(double rho0, double cs2, double kT, double kappa, double ta
         sL[j][0] = 0.25 * l11; sL[j][1] = 0.0;
         sL[j][2] = 0.25 * l21; sL[j][3] = 0.25 * l22;
     }
-    pair_stencil(sL, c, rec);
+    pair_stencil(sL, rec);
     rec->mode = (noise_mode == LB_NOISE_OFF || kT <= 0.0)
                     ? 0
                     : (noise_mode == LB_NOISE_FULL ? 2 : (noise_mode == LB_NOISE_FULL_RS ? 3 : 1));

@@ -457,17 +457,18 @@ cudaError_t launch_step_simple(const StepArgs& a, int noise_mode, int fp16, cuda
 cudaError_t launch_step_simple_d(const StepArgsD& a, int noise_mode, cudaStream_t s);
 cudaError_t launch_step_sweep(const StepArgs& a, int noise_mode, int fp16, int occ6, cudaStream_t s);
 bool sweep_fits(const Grid& g);
-cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* src_map, const void* dst_map, int* err, int noise_mode, int tile, int fp16,
+cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* src_map, const void* dst_map, int* err, int noise_mode, int tile,
                             cudaStream_t s, bool poly = false);
+cudaError_t launch_step_half(const StepArgs& a, const void* src_map, int* err, int noise_mode, int tile, cudaStream_t s);
 bool make_pop_tensor_maps(const void* buf, const Grid& g, int tile, int fp16, void* load_map, void* store_map);
 int tma_tile_count();
 int tma_default_tile(int noise_mode, int fp16);
 size_t tensor_map_bytes();
-// many steps of a small lattice in one launch (lb_step_resident.cu)
+// many steps of a small FP32 lattice in one launch (lb_step_resident.cu)
 bool resident_fits(const Grid& g);
 bool resident_available();
-cudaError_t launch_step_resident(const StepArgs& a, const StepArgsD& d, long long t, int nsteps, int noise_mode, int fp16,
-                                 bool poly, cudaStream_t s);
+cudaError_t launch_step_resident(const StepArgs& a, const StepArgsD& d, long long t, int nsteps, int noise_mode, bool poly,
+                                 cudaStream_t s);
 cudaError_t launch_noise49(float2* buf, float2* scratch, const NoiseGenArgs& ga, const float2* twx,
                            const float2* twy, cudaStream_t s);
 cudaError_t launch_noise49_d(double2* buf, const NoiseGenArgsD& ga, const double2* twx, const double2* twy,

@@ -1,10 +1,9 @@
 // lb_pair.cuh -- the fluctuating collision of two nodes side by side, for the TMA-staged step
-// kernels (single lattice, batched ensemble, server).
+// kernels of FP32 storage (single lattice, batched ensemble, server).
 //
 // What bounds a step.  At 72 bytes a node the 4096^2 step cannot take less than 178 us (copy
 // bandwidth 6790 GB/s); with one node per arithmetic instruction it took 212 us, because a node
-// cost 341 issued instructions at 68 % issue (FP16 storage: 368 instructions and 220 us for half
-// the bytes).  So this file spends fewer instructions per node:
+// cost 341 issued instructions at 68 % issue.  So this file spends fewer instructions per node:
 //   * a thread's nodes are pairs (x, x + 1), x even, and the FP32 arithmetic is on packed pairs
 //     (add, mul, fma .f32x2: one issue slot for two nodes; the FMA pipe runs them at the same
 //     128 operations a clock per SM as scalar ones, measured 120, and 80 when all three operands
@@ -12,7 +11,7 @@
 //     the constant bank, which cost nothing as a broadcast operand);
 //   * rows of a thread's pairs are adjacent, so the density rows of its stencils are loaded once
 //     (12 shared loads for 2 x 2 nodes instead of 36) and their sums over x are shared;
-//   * planes with c_x = 0, the density and all stores move 8 bytes (FP16: 4) at a time;
+//   * planes with c_x = 0, the density and all stores move 8 bytes at a time;
 //   * the relaxation and noise factors carry the 1/N_a and w_i of the back-transform (host side,
 //     PairCoef), and the stencil weights 1/6 and 1/12 are folded into kappa;
 //   * log2, sine and cosine are the flush-to-zero forms (their arguments are never subnormal),
@@ -81,11 +80,12 @@ __device__ __forceinline__ void gauss2(uint32_t wa, uint32_t wb, F2* n0, F2* n1)
 
 // --- coefficients ----------------------------------------------------------------------------
 
-// One lattice's coefficients as collide_pair takes them.  c = 1/36 (populations stored as
-// deviations df_i: the diagonal weight; the axis and rest weights are then 4 c and 16 c) or 1
-// (stored g_i = df_i / w_i).  A mode's increment enters the back-transform as c D_a / N_a times
-// the common factors 1 (a = 4), 1 (5), 1 (6), 1 (7, 8), 1 (9) of collide_node's d4..d9; noise
-// factors carry GAUSS_SCALE as well (G below).
+// One lattice's coefficients as collide_pair takes them, with c = 1/36 (the diagonal weight; the
+// axis and rest weights are 4 c and 16 c).  A mode's increment enters the back-transform as
+// c D_a / N_a times the common factors 1 (a = 4), 1 (5), 1 (6), 1 (7, 8), 1 (9) of collide_node's
+// d4..d9; noise factors carry GAUSS_SCALE as well (G below).
+constexpr double PAIR_SCALE = 1.0 / 36.0;
+
 struct PairCoef {
     float rho0, cs2m;
     float kl, kg;                    // -kappa / 6 and kappa / 144
@@ -110,7 +110,8 @@ struct PairStencil {
 
 template <typename S>
 __host__ inline void pair_coef(double rho0, double cs2m, double kappa, double lb, double ls, double lq, double le,
-                               const S L[4], const S s[3], double c, PairCoef* o) {
+                               const S L[4], const S s[3], PairCoef* o) {
+    const double c = PAIR_SCALE;
     o->rho0 = (float)rho0;
     o->cs2m = (float)cs2m;
     o->kl = (float)(-kappa / 6.0);
@@ -133,8 +134,8 @@ __host__ inline void pair_coef(double rho0, double cs2m, double kappa, double lb
 }
 
 template <typename S>
-__host__ inline void pair_stencil(const S sL[3][4], double c, PairStencil* o) {
-    const double G = GAUSS_SCALE * c;
+__host__ inline void pair_stencil(const S sL[3][4], PairStencil* o) {
+    const double G = GAUSS_SCALE * PAIR_SCALE;
     for (int j = 0; j < 3; ++j) {
         o->sL[j][0] = (float)(G * sL[j][0] / 4.0);
         o->sL[j][1] = (float)(G * sL[j][1] / 4.0);
@@ -144,7 +145,8 @@ __host__ inline void pair_stencil(const S sL[3][4], double c, PairStencil* o) {
 }
 
 template <typename S>
-__host__ inline void pair_local(double e2, double e3, double e4, const S cq[4], const S lu[9], double c, PairLocal* o) {
+__host__ inline void pair_local(double e2, double e3, double e4, const S cq[4], const S lu[9], PairLocal* o) {
+    const double c = PAIR_SCALE;
     o->e2 = (float)e2;
     o->e3 = (float)e3;
     o->e4 = (float)e4;
@@ -154,22 +156,14 @@ __host__ inline void pair_local(double e2, double e3, double e4, const S cq[4], 
     for (int q = 0; q < 9; ++q) o->lu[q] = (float)(f[q] * lu[q]);
 }
 
-// scale c of a storage type's coefficients
-template <bool GF>
-constexpr double pair_scale() { return GF ? 1.0 : 1.0 / 36.0; }
-
 // --- one pair --------------------------------------------------------------------------------
 
 // density deviation of a pair from its pulled values (one order of summation, for a node and for
-// the ring: drho_of / drho_of_g of lb_collide.cuh are the scalar counterparts)
-template <bool GF>
+// the ring: drho_of of lb_collide.cuh is the scalar counterpart)
 __device__ __forceinline__ F2 drho_pair(const F2 f[Q]) {
     const F2 sa = add2(add2(f[1], f[3]), add2(f[2], f[4]));
     const F2 sd = add2(add2(f[5], f[7]), add2(f[6], f[8]));
-    if constexpr (GF)
-        return fma2(bc(4.0f / 9.0f), f[0], fma2(bc(1.0f / 9.0f), sa, mul2(bc(1.0f / 36.0f), sd)));
-    else
-        return add2(add2(f[0], sa), sd);
+    return add2(add2(f[0], sa), sd);
 }
 
 // The stencil of a pair: 6 lap rho, 12 d_x rho, 12 d_y rho (Appendix B and the isotropic
@@ -193,30 +187,18 @@ __device__ __forceinline__ RhoRow rho_row(const float* R) {
 // its stencil; node: the first node's index (the second's is node + 1); z4, z9: the scaled
 // (xi_4, xi_9) of modes 2 and 3; a: coefficients (PairCoef, the round keys rk and the time t_lo,
 // t_hi); loc: POLY and MODE 4.  Writes the nine post-collision values of both nodes.
-template <int MODE, bool POLY, bool GF, typename Args>
+template <int MODE, bool POLY, typename Args>
 __device__ __forceinline__ void collide_pair(const Args& a, const PairLocal* loc, const F2 f[Q], F2 rho, F2 lap6,
                                              F2 gx12, F2 gy12, uint32_t node, F2 z4, F2 z9, F2 o[Q]) {
     // moments of the deviations (rows of T, Eq. Tmat); ux of opposite pairs first
-    F2 g0 = f[0];
-    F2 sa = add2(add2(f[1], f[3]), add2(f[2], f[4]));
-    F2 sd = add2(add2(f[5], f[7]), add2(f[6], f[8]));
-    F2 nax = sub2(f[3], f[1]), nay = sub2(f[4], f[2]);                   // minus the axis momenta
+    const F2 g0 = f[0];
+    const F2 sa = add2(add2(f[1], f[3]), add2(f[2], f[4]));
+    const F2 sd = add2(add2(f[5], f[7]), add2(f[6], f[8]));
+    const F2 nax = sub2(f[3], f[1]), nay = sub2(f[4], f[2]);             // minus the axis momenta
     const F2 d57 = sub2(f[5], f[7]), d86 = sub2(f[8], f[6]);
-    F2 dx = add2(d57, d86), dy = sub2(d57, d86);
-    F2 m5 = sub2(add2(f[1], f[3]), add2(f[2], f[4]));
-    F2 m6 = sub2(add2(f[5], f[7]), add2(f[6], f[8]));
-    if constexpr (GF) {
-        const F2 wa = bc(1.0f / 9.0f), wd = bc(1.0f / 36.0f);
-        g0 = mul2(g0, bc(4.0f / 9.0f));
-        sa = mul2(sa, wa);
-        sd = mul2(sd, wd);
-        nax = mul2(nax, wa);
-        nay = mul2(nay, wa);
-        dx = mul2(dx, wd);
-        dy = mul2(dy, wd);
-        m5 = mul2(m5, wa);
-        m6 = mul2(m6, wd);
-    }
+    const F2 dx = add2(d57, d86), dy = sub2(d57, d86);
+    const F2 m5 = sub2(add2(f[1], f[3]), add2(f[2], f[4]));
+    const F2 m6 = sub2(add2(f[5], f[7]), add2(f[6], f[8]));
     const F2 jx = sub2(dx, nax), jy = sub2(dy, nay);
     const F2 m4 = fma2(sd, bc(4.0f), fma2(g0, bc(-2.0f), sa));
     const F2 m9 = fma2(sd, bc(8.0f), fma2(sa, bc(-4.0f), add2(g0, g0)));
@@ -304,19 +286,11 @@ __device__ __forceinline__ void collide_pair(const Args& a, const PairLocal* loc
     o[7] = add2(f[7], fma2(p, bc(-2.0f), D1));
     o[6] = add2(f[6], fma2(m, bc(-2.0f), D2));
     o[8] = add2(f[8], fma2(m, bc(2.0f), D2));
-    if constexpr (GF) {
-        o[0] = fma2(sub2(d9, d4), bc(2.0f), f[0]);
-        o[1] = add2(f[1], sub2(A1, d7));
-        o[2] = add2(f[2], sub2(A2, d8));
-        o[3] = add2(f[3], add2(A1, d7));
-        o[4] = add2(f[4], add2(A2, d8));
-    } else {
-        o[0] = fma2(sub2(d9, d4), bc(32.0f), f[0]);
-        o[1] = fma2(sub2(A1, d7), bc(4.0f), f[1]);
-        o[2] = fma2(sub2(A2, d8), bc(4.0f), f[2]);
-        o[3] = fma2(add2(A1, d7), bc(4.0f), f[3]);
-        o[4] = fma2(add2(A2, d8), bc(4.0f), f[4]);
-    }
+    o[0] = fma2(sub2(d9, d4), bc(32.0f), f[0]);
+    o[1] = fma2(sub2(A1, d7), bc(4.0f), f[1]);
+    o[2] = fma2(sub2(A2, d8), bc(4.0f), f[2]);
+    o[3] = fma2(add2(A1, d7), bc(4.0f), f[3]);
+    o[4] = fma2(add2(A2, d8), bc(4.0f), f[4]);
 }
 
 // --- a staged tile ------------------------------------------------------------------------------
@@ -342,16 +316,10 @@ constexpr int pair_min_blocks() {
 
 // The pulled values of the pair whose unshifted box index is b (even): plane i at b - cx_i, the
 // y shift already in the box origin.
-template <int PS, bool GF, typename T>
-__device__ __forceinline__ void pull_pair(const T* S, int b, F2 f[Q]) {
-    auto even = [&](int i, int k) -> F2 {
-        if constexpr (GF) return __half22float2(*reinterpret_cast<const __half2*>(S + i * PS + k));
-        else return *reinterpret_cast<const F2*>(S + i * PS + k);
-    };
-    auto odd = [&](int i, int k) -> F2 {
-        if constexpr (GF) return make_float2(__half2float(S[i * PS + k]), __half2float(S[i * PS + k + 1]));
-        else return make_float2(S[i * PS + k], S[i * PS + k + 1]);
-    };
+template <int PS>
+__device__ __forceinline__ void pull_pair(const float* S, int b, F2 f[Q]) {
+    auto even = [&](int i, int k) -> F2 { return *reinterpret_cast<const F2*>(S + i * PS + k); };
+    auto odd = [&](int i, int k) -> F2 { return make_float2(S[i * PS + k], S[i * PS + k + 1]); };
     f[0] = even(0, b);
     f[1] = odd(1, b - 1);
     f[2] = even(2, b);
@@ -370,17 +338,17 @@ __device__ __forceinline__ void pull_pair(const T* S, int b, F2 f[Q]) {
 // instructions on 6 of 16 warps of a 64 x 16 tile, this one 30 on 4); FIRST puts them on the first
 // threads instead, where the last form the noise contributions of the halo.  Nodes beyond a ragged
 // edge take part (their values are never used).
-template <int TX, int TY, int NT, bool GF, bool FIRST, typename T>
-__device__ __forceinline__ void tile_pull(const T* S, float* R, F2 (&fr)[PairMap<TX, TY, NT>::RPT][Q]) {
-    using TT = TmaTile<TX, TY, T>;
+template <int TX, int TY, int NT, bool FIRST>
+__device__ __forceinline__ void tile_pull(const float* S, float* R, F2 (&fr)[PairMap<TX, TY, NT>::RPT][Q]) {
+    using TT = TmaTile<TX, TY>;
     using M = PairMap<TX, TY, NT>;
     const int tid = threadIdx.x;
     const int lx = 2 * (tid % M::PX), ly = (tid / M::PX) * M::RPT;
     if (M::ACTIVE == NT || tid < M::ACTIVE) {
 #pragma unroll
         for (int j = 0; j < M::RPT; ++j) {
-            pull_pair<TT::PS, GF>(S, (ly + j + 1) * TT::BW + lx + TT::XO, fr[j]);
-            *reinterpret_cast<F2*>(R + (ly + j + 1) * TT::RW + lx + 2) = drho_pair<GF>(fr[j]);
+            pull_pair<TT::PS>(S, (ly + j + 1) * TT::BW + lx + TT::XO, fr[j]);
+            *reinterpret_cast<F2*>(R + (ly + j + 1) * TT::RW + lx + 2) = drho_pair(fr[j]);
         }
     }
     constexpr int NR = TX, NC = 2 * (TY + 2);          // row pairs (below, then above); column nodes
@@ -388,23 +356,15 @@ __device__ __forceinline__ void tile_pull(const T* S, float* R, F2 (&fr)[PairMap
         if (j < NR) {
             const int p = 2 * (j % M::PX), ry = j < M::PX ? 0 : TY + 1;
             F2 f[Q];
-            pull_pair<TT::PS, GF>(S, ry * TT::BW + p + TT::XO, f);
-            *reinterpret_cast<F2*>(R + ry * TT::RW + p + 2) = drho_pair<GF>(f);
+            pull_pair<TT::PS>(S, ry * TT::BW + p + TT::XO, f);
+            *reinterpret_cast<F2*>(R + ry * TT::RW + p + 2) = drho_pair(f);
         } else {
             const int u = j - NR, ry = u >> 1, rx = (u & 1) ? TX : -1;
             const int b = ry * TT::BW + rx + TT::XO;
-            auto at = [&](int i, int k) -> float {
-                if constexpr (GF) return __half2float(S[i * TT::PS + k]);
-                else return S[i * TT::PS + k];
-            };
+            auto at = [&](int i, int k) -> float { return S[i * TT::PS + k]; };
             const float sa = (at(1, b - 1) + at(3, b + 1)) + (at(2, b) + at(4, b));
             const float sd = (at(5, b - 1) + at(7, b + 1)) + (at(6, b + 1) + at(8, b - 1));
-            float v;
-            if constexpr (GF)
-                v = fmaf(4.0f / 9.0f, at(0, b), fmaf(1.0f / 9.0f, sa, __fmul_rn(1.0f / 36.0f, sd)));
-            else
-                v = (at(0, b) + sa) + sd;
-            R[ry * TT::RW + rx + 2] = v;
+            R[ry * TT::RW + rx + 2] = (at(0, b) + sa) + sd;
         }
     }
 }
@@ -516,27 +476,21 @@ __device__ __forceinline__ void stencil_tile(const Args& a, unsigned char* x, in
 // Whether the tile at x0 is stored by its threads instead of its TMA box: a box is clipped at the
 // lattice's last column in units of 16 bytes, so a row that ends inside such a unit would lose its
 // first ghost columns to the tile's unused ones.
-template <int TX, typename T>
+template <int TX>
 __device__ __forceinline__ bool tile_direct(const Grid& g, int x0) {
-    return x0 + TX > g.nx && g.nx % Elem<T>::XO != 0;
+    return x0 + TX > g.nx && g.nx % Elem<float>::XO != 0;
 }
 
-// a pair in the storage type, at an even column
-template <bool GF, typename T>
-__device__ __forceinline__ void put_pair(T* q, F2 v) {
-    if constexpr (GF) *reinterpret_cast<__half2*>(q) = __floats2half2_rn(v.x, v.y);
-    else *reinterpret_cast<F2*>(q) = v;
-}
+// a pair, at an even column
+__device__ __forceinline__ void put_pair(float* q, F2 v) { *reinterpret_cast<F2*>(q) = v; }
 
 // the nodes of the pair at (x, y) themselves (a tile that tile_direct names); the second only if
 // x + 1 < nx
-template <typename T, bool GF>
-__device__ __forceinline__ void store_pair(T* dst, long long P, const Grid& g, int x, int y, const F2 o[Q]) {
-    T* p = dst + g.at(x, y);
+__device__ __forceinline__ void store_pair(float* dst, long long P, const Grid& g, int x, int y, const F2 o[Q]) {
+    float* p = dst + g.at(x, y);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        if (x + 1 < g.nx) put_pair<GF>(p + i * P, o[i]);
-        else if constexpr (GF) p[i * P] = Elem<T>::store_g(o[i].x);
+        if (x + 1 < g.nx) put_pair(p + i * P, o[i]);
         else p[i * P] = o[i].x;
     }
 }
@@ -545,31 +499,30 @@ __device__ __forceinline__ void store_pair(T* dst, long long P, const Grid& g, i
 // lb_internal.cuh); the nodes themselves leave with the tile.  Where nx is even and no node feeds
 // more than one ghost column and row, both nodes of a pair feed the same ones and the copies are
 // pairs; else each node is written with all its copies.
-template <typename T, bool GF>
-__device__ __forceinline__ void ghost_pair(T* dst, long long P, const Grid& g, int x, int y, const F2 o[Q]) {
-    constexpr int GW = Elem<T>::GW;
+__device__ __forceinline__ void ghost_pair(float* dst, long long P, const Grid& g, int x, int y, const F2 o[Q]) {
+    constexpr int GW = Elem<float>::GW;
     if (!(x < GW || x + 1 >= g.nx - GW || y < 2 || y >= g.ny - 2)) return;
     if ((g.nx & 1) == 0 && g.nx >= 2 * GW && g.ny >= 4) {
-        T* p = dst + g.at(x, y);
+        float* p = dst + g.at(x, y);
         const bool hx = x < GW || x >= g.nx - GW, hy = y < 2 || y >= g.ny - 2;
         const long long dx = x < GW ? (long long)g.nx : -(long long)g.nx;
         const long long dy = (y < 2 ? (long long)g.ny : -(long long)g.ny) * g.pitch;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            T* q = p + i * P;
-            if (hx) put_pair<GF>(q + dx, o[i]);
-            if (hy) put_pair<GF>(q + dy, o[i]);
-            if (hx & hy) put_pair<GF>(q + dx + dy, o[i]);
+            float* q = p + i * P;
+            if (hx) put_pair(q + dx, o[i]);
+            if (hy) put_pair(q + dy, o[i]);
+            if (hx & hy) put_pair(q + dx + dy, o[i]);
         }
     } else {
         float v[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) v[i] = o[i].x;
-        store9<T, float, GF>(dst, P, g, x, y, v);
+        store9<float, float>(dst, P, g, x, y, v);
         if (x + 1 < g.nx) {
 #pragma unroll
             for (int i = 0; i < Q; ++i) v[i] = o[i].y;
-            store9<T, float, GF>(dst, P, g, x + 1, y, v);
+            store9<float, float>(dst, P, g, x + 1, y, v);
         }
     }
 }
@@ -577,15 +530,15 @@ __device__ __forceinline__ void ghost_pair(T* dst, long long P, const Grid& g, i
 // After the tile's barrier: collide the thread's nodes from the pulled values fr and the density
 // tile R into the outgoing tile `out` (one TMA store per tile takes it away: nine 8-byte shared
 // stores at fixed offsets from one address in place of nine global ones with an address each), and
-// write the ghost copies of a tile near an edge to dst.  xi49: the (xi_4, xi_9) field of MODE 2 (nx even there); z4, z9 and x: the in-block
-// sums and the exchange of MODE 3.
-template <int MODE, bool POLY, bool GF, int TX, int TY, int NT, typename T, typename Args>
+// write the ghost copies of a tile near an edge to dst.  xi49: the (xi_4, xi_9) field of MODE 2 (nx even
+// there); z4, z9 and xch: the in-block sums and the exchange of MODE 3.
+template <int MODE, bool POLY, int TX, int TY, int NT, typename Args>
 __device__ __forceinline__ void tile_collide(const Args& a, const PairLocal* loc,
                                              const F2 (&fr)[PairMap<TX, TY, NT>::RPT][Q], const float* R,
-                                             const Grid& g, int x0, int y0, T* out, T* dst, const float2* __restrict__ xi49,
+                                             const Grid& g, int x0, int y0, float* out, float* dst, const float2* __restrict__ xi49,
                                              const F2 (&z4)[PairMap<TX, TY, NT>::RPT],
                                              const F2 (&z9)[PairMap<TX, TY, NT>::RPT], const unsigned char* xch) {
-    using TT = TmaTile<TX, TY, T>;
+    using TT = TmaTile<TX, TY>;
     using M = PairMap<TX, TY, NT>;
     using ST = StencilTile<TX, TY, NT>;
     const int tid = threadIdx.x;
@@ -593,9 +546,9 @@ __device__ __forceinline__ void tile_collide(const Args& a, const PairLocal* loc
     const int lx = 2 * p, ly = rb * M::RPT;
     const int x = x0 + lx;
     if ((M::ACTIVE < NT && tid >= M::ACTIVE) || x >= g.nx || y0 + ly >= g.ny) return;
-    const bool edge = x0 < Elem<T>::GW || x0 + TX > g.nx - Elem<T>::GW || y0 < 2 || y0 + TY > g.ny - 2;
+    const bool edge = x0 < Elem<float>::GW || x0 + TX > g.nx - Elem<float>::GW || y0 < 2 || y0 + TY > g.ny - 2;
     const float* r0 = R + (ly + 1) * TT::RW + lx + 2;
-    T* po = out + ly * TX + lx;
+    float* po = out + ly * TX + lx;
     RhoRow m = rho_row(r0 - TT::RW), c = rho_row(r0);
 #pragma unroll
     for (int j = 0; j < M::RPT; ++j) {
@@ -626,11 +579,11 @@ __device__ __forceinline__ void tile_collide(const Args& a, const PairLocal* loc
             v9.x += e.y + q.y;
         }
         F2 o[Q];
-        collide_pair<MODE, POLY, GF>(a, loc, fr[j], c.C, lap6, gx12, gy12, node, v4, v9, o);
+        collide_pair<MODE, POLY>(a, loc, fr[j], c.C, lap6, gx12, gy12, node, v4, v9, o);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) put_pair<GF>(po + (i * TY + j) * TX, o[i]);
-        if (edge && tile_direct<TX, T>(g, x0)) store_pair<T, GF>(dst, g.plane, g, x, y, o);
-        if (edge) ghost_pair<T, GF>(dst, g.plane, g, x, y, o);
+        for (int i = 0; i < Q; ++i) put_pair(po + (i * TY + j) * TX, o[i]);
+        if (edge && tile_direct<TX>(g, x0)) store_pair(dst, g.plane, g, x, y, o);
+        if (edge) ghost_pair(dst, g.plane, g, x, y, o);
         m = c;
         c = n;
     }

@@ -63,7 +63,7 @@ constexpr int SV_GX = 32;            // ghost columns per side of every served l
 // its dynamic shared memory
 template <bool RS>
 constexpr int serve_smem() {
-    return TmaTile<SV_TX, SV_TY, float>::SMEM_BYTES + (RS ? StencilTile<SV_TX, SV_TY, SV_NT>::BYTES : 0);
+    return TmaTile<SV_TX, SV_TY>::SMEM_BYTES + (RS ? StencilTile<SV_TX, SV_TY, SV_NT>::BYTES : 0);
 }
 
 // index of the active slot that owns `tile`: the last a with tile_begin[a] <= tile
@@ -93,7 +93,7 @@ __global__ void serve_tiles_kernel(const ServeParams p, int tx, int ty) {
 // for chunks that hold one; its extra path raises the register count)
 template <int TX, int TY, int NT, bool RS>
 __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_serve_kernel(const ServeParams p) {
-    using TT = TmaTile<TX, TY, float>;
+    using TT = TmaTile<TX, TY>;
     using M = PairMap<TX, TY, NT>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float* S = reinterpret_cast<float*>(smem_raw);
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
     auto store = [&](int s) {
         Grid g;
         g.nx = __ldg(&p.desc[st_slot[s]].g.nx);
-        if (tile_direct<TX, float>(g, st_x0[s])) return;
+        if (tile_direct<TX>(g, st_x0[s])) return;
         tma_store_3d(smap, smem_u32(out), st_x0[s], st_y0[s], 0);
         tma_store_commit();
     };
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
         // pulled populations stay in registers across the density barrier; the next tile is
         // loaded right after it (the other turn's slot and origin, read by the store above, are free)
         F2 fr[M::RPT][Q], z4[M::RPT], z9[M::RPT];
-        tile_pull<TX, TY, NT, false, RS>(S, R, fr);
+        tile_pull<TX, TY, NT, RS>(S, R, fr);
         if (tid == 0) tma_store_wait_read();
         __syncthreads();
         const int mode = sargs.mode;        // the tile's: uniform over the CTA
@@ -199,17 +199,17 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
             if (mode == 3) {
                 stencil_tile<TX, TY, NT>(sargs, xch, x0, y0, g.nx, g.ny, z4, z9);
                 __syncthreads();
-                tile_collide<3, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, xch);
+                tile_collide<3, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, xch);
                 stepped = true;
             }
         }
         if (!stepped) {
             if (mode == 2)
-                tile_collide<2, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, d->xi, z4, z9, nullptr);
+                tile_collide<2, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, d->xi, z4, z9, nullptr);
             else if (mode)
-                tile_collide<1, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, nullptr);
+                tile_collide<1, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, nullptr);
             else
-                tile_collide<0, false, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, nullptr);
+                tile_collide<0, false, TX, TY, NT>(sargs, nullptr, fr, R, g, x0, y0, out, dst, nullptr, z4, z9, nullptr);
         }
         fence_async_smem();
     }
@@ -931,7 +931,7 @@ int lb_server_create(size_t hbm_budget_bytes, int max_active, int max_chunk_step
     if ((e = cudaMemset(s->d_k, 0, sizeof(long long))) != cudaSuccess) return fail_create(e);
     if ((e = cudaMemset(s->d_done, 0, sizeof(unsigned int))) != cudaSuccess) return fail_create(e);
     if ((e = cudaMemset(s->d_err, 0, sizeof(int))) != cudaSuccess) return fail_create(e);
-    using TT = TmaTile<SV_TX, SV_TY, float>;
+    using TT = TmaTile<SV_TX, SV_TY>;
     auto kern = step_serve_kernel<SV_TX, SV_TY, SV_NT, false>;
     auto kern_rs = step_serve_kernel<SV_TX, SV_TY, SV_NT, true>;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, serve_smem<false>())) != cudaSuccess)

@@ -1,4 +1,4 @@
-// lb_step_resident.cu -- many steps of a small D2Q9 lattice in one launch, its populations resident in
+// lb_step_resident.cu -- many steps of a small FP32 D2Q9 lattice in one launch, its populations resident in
 // the shared memory of a cluster of CTAs.
 //
 // A step of a lattice of up to 128^2 nodes is all latency: launched one by one it takes 3.8 us (launch,
@@ -15,7 +15,6 @@
 #include <cooperative_groups.h>
 
 #include <atomic>
-#include <type_traits>
 
 #include "lb_pair.cuh"
 
@@ -34,8 +33,8 @@ struct ResArgs {
     ResCoef c;
     PairLocal loc;
     Grid g;
-    const void* src;
-    void* dst;
+    const float* src;
+    float* dst;
     long long t;
     int steps;
     int pw, ps;        // elements per stored row (nx + 8) and per plane
@@ -43,13 +42,11 @@ struct ResArgs {
 };
 
 // bytes of the two population buffers; the density tile follows
-template <typename T>
-__host__ __device__ inline int res_buf_bytes(const ResArgs& a) { return 2 * Q * a.ps * (int)sizeof(T); }
+__host__ __device__ inline int res_buf_bytes(const ResArgs& a) { return 2 * Q * a.ps * (int)sizeof(float); }
 
-template <int MODE, bool POLY, typename T>
+template <int MODE, bool POLY>
 __global__ void __launch_bounds__(RES_MAX_NX / 2 * 10) step_resident_kernel(const __grid_constant__ ResArgs a) {
     namespace cg = cooperative_groups;
-    constexpr bool GF = std::is_same<T, __half>::value;
     extern __shared__ __align__(16) unsigned char res_smem[];
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
@@ -58,20 +55,20 @@ __global__ void __launch_bounds__(RES_MAX_NX / 2 * 10) step_resident_kernel(cons
     const int y0 = rank * ny / RES_CTAS, rows = (rank + 1) * ny / RES_CTAS - y0;
     const int below = (rank + RES_CTAS - 1) % RES_CTAS, above = (rank + 1) % RES_CTAS;
     const int rows_below = (below + 1) * ny / RES_CTAS - below * ny / RES_CTAS;
-    T* buf = reinterpret_cast<T*>(res_smem);               // [2][Q][rows + 4][pw], node (x, r) at (r + 2) pw + x + 4
-    float* R = reinterpret_cast<float*>(res_smem + res_buf_bytes<T>(a));   // node (x, r) at (r + 1)(nx + 4) + x + 2
+    float* buf = reinterpret_cast<float*>(res_smem);           // [2][Q][rows + 4][pw], node (x, r) at (r + 2) pw + x + 4
+    float* R = reinterpret_cast<float*>(res_smem + res_buf_bytes(a));   // node (x, r) at (r + 1)(nx + 4) + x + 2
     const int tid = threadIdx.x, rw = nx + 4;
 
     // the band and its halo from the stored planes (columns -2 .. nx + 1, rows -2 .. rows + 1)
     {
-        const T* src = static_cast<const T*>(a.src);
+        const float* src = a.src;
         const int w = hx + 2, n = w * (rows + 4);
         for (int e = tid; e < n; e += blockDim.x) {
             const int r = e / w, x = 2 * (e - r * w) - 2;
             const long long o = g.at(x, y0 + r - 2);
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
-                T* d = buf + i * ps + r * pw + x + 4;
+                float* d = buf + i * ps + r * pw + x + 4;
                 d[0] = src[i * g.plane + o];
                 d[1] = src[i * g.plane + o + 1];
             }
@@ -96,26 +93,25 @@ __global__ void __launch_bounds__(RES_MAX_NX / 2 * 10) step_resident_kernel(cons
     const uint32_t node = (uint32_t)y * (uint32_t)nx + (uint32_t)x;
     // offsets of the pair in the halo rows of the neighbours that hold a copy of it (rows >= 2)
     const bool to_below = own && r < 2, to_above = own && r >= rows - 2;
-    T* const nb_below = cluster.map_shared_rank(buf, below);
-    T* const nb_above = cluster.map_shared_rank(buf, above);
+    float* const nb_below = cluster.map_shared_rank(buf, below);
+    float* const nb_above = cluster.map_shared_rank(buf, above);
     const int at_below = (rows_below + r + 2) * pw + x + 4, at_above = (r - rows + 2) * pw + x + 4;
     const int wrap = x < 2 ? nx : (x >= nx - 2 ? -nx : 0);
     cluster.sync();        // every CTA runs and has loaded its band
 
     ResCoef c = a.c;
     for (int k = 0; k < a.steps; ++k) {
-        const T* S = buf + (k & 1) * Q * ps;
+        const float* S = buf + (k & 1) * Q * ps;
         const int to = ((k & 1) ^ 1) * Q * ps;
         F2 f[Q];
         if (own || ring) {
             constexpr int cx[Q] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, cy[Q] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
-                const T* s = S + i * ps + at - cy[i] * pw - cx[i];
-                if constexpr (GF) f[i] = make_float2(__half2float(s[0]), __half2float(s[1]));
-                else f[i] = make_float2(s[0], s[1]);
+                const float* s = S + i * ps + at - cy[i] * pw - cx[i];
+                f[i] = make_float2(s[0], s[1]);
             }
-            const F2 rho = drho_pair<GF>(f);
+            const F2 rho = drho_pair(f);
             *reinterpret_cast<F2*>(pr) = rho;
             if (x == 0) pr[nx] = rho.x;                    // column nx
             if (x == nx - 2) pr[1 - nx] = rho.y;           // column -1
@@ -130,33 +126,33 @@ __global__ void __launch_bounds__(RES_MAX_NX / 2 * 10) step_resident_kernel(cons
             const F2 gx12 = fma2(d.d, bc(4.0f), add2(n.d, m.d));
             const F2 gy12 = fma2(sub2(n.C, m.C), bc(4.0f), sub2(n.s, m.s));
             F2 o[Q];
-            collide_pair<MODE, POLY, GF>(c, &a.loc, f, d.C, lap6, gx12, gy12, node, bc(0.f), bc(0.f), o);
+            collide_pair<MODE, POLY>(c, &a.loc, f, d.C, lap6, gx12, gy12, node, bc(0.f), bc(0.f), o);
             if (k + 1 < a.steps) {
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
-                    T* q = buf + to + i * ps + at;
-                    put_pair<GF>(q, o[i]);
-                    if (wrap) put_pair<GF>(q + wrap, o[i]);
+                    float* q = buf + to + i * ps + at;
+                    put_pair(q, o[i]);
+                    if (wrap) put_pair(q + wrap, o[i]);
                 }
                 if (to_below) {
 #pragma unroll
                     for (int i = 0; i < Q; ++i) {
-                        T* q = nb_below + to + i * ps + at_below;
-                        put_pair<GF>(q, o[i]);
-                        if (wrap) put_pair<GF>(q + wrap, o[i]);
+                        float* q = nb_below + to + i * ps + at_below;
+                        put_pair(q, o[i]);
+                        if (wrap) put_pair(q + wrap, o[i]);
                     }
                 }
                 if (to_above) {
 #pragma unroll
                     for (int i = 0; i < Q; ++i) {
-                        T* q = nb_above + to + i * ps + at_above;
-                        put_pair<GF>(q, o[i]);
-                        if (wrap) put_pair<GF>(q + wrap, o[i]);
+                        float* q = nb_above + to + i * ps + at_above;
+                        put_pair(q, o[i]);
+                        if (wrap) put_pair(q + wrap, o[i]);
                     }
                 }
             } else {
-                store_pair<T, GF>(static_cast<T*>(a.dst), g.plane, g, x, y, o);
-                ghost_pair<T, GF>(static_cast<T*>(a.dst), g.plane, g, x, y, o);
+                store_pair(a.dst, g.plane, g, x, y, o);
+                ghost_pair(a.dst, g.plane, g, x, y, o);
             }
         }
         // every CTA's stores into this one's next buffer are done and visible, and this one's reads of
@@ -173,9 +169,9 @@ bool resident_fits(const Grid& g) {
     return g.nx % 2 == 0 && g.nx >= 32 && g.nx <= RES_MAX_NX && g.ny >= 2 * RES_CTAS && g.ny <= 8 * RES_CTAS;
 }
 
-template <int MODE, bool POLY, typename T>
+template <int MODE, bool POLY>
 static cudaError_t launch_res(const ResArgs& a, int threads, size_t smem, cudaStream_t s) {
-    auto kern = step_resident_kernel<MODE, POLY, T>;
+    auto kern = step_resident_kernel<MODE, POLY>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -194,15 +190,6 @@ static cudaError_t launch_res(const ResArgs& a, int threads, size_t smem, cudaSt
     return cudaLaunchKernelEx(&c, kern, a);
 }
 
-template <typename T>
-static cudaError_t launch_res_t(const ResArgs& a, int noise_mode, bool poly, int threads, size_t smem, cudaStream_t s) {
-    switch (noise_mode) {
-        case 0: return poly ? launch_res<0, true, T>(a, threads, smem, s) : launch_res<0, false, T>(a, threads, smem, s);
-        case 1: return poly ? launch_res<1, true, T>(a, threads, smem, s) : launch_res<1, false, T>(a, threads, smem, s);
-        default: return poly ? launch_res<4, true, T>(a, threads, smem, s) : launch_res<4, false, T>(a, threads, smem, s);
-    }
-}
-
 // Whether this device can hold such a cluster at its largest (a launch that it cannot hold is refused);
 // asked once per device.
 bool resident_available() {
@@ -211,7 +198,7 @@ bool resident_available() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return false;
     int k = known[dev].load(std::memory_order_acquire);
     if (k == 0) {
-        auto kern = step_resident_kernel<1, false, float>;
+        auto kern = step_resident_kernel<1, false>;
         const int smem = 2 * Q * (RES_MAX_NX + 8) * 12 * 4 + 10 * (RES_MAX_NX + 4) * 4;
         cudaLaunchConfig_t c = {};
         c.gridDim = dim3(RES_CTAS);
@@ -235,18 +222,17 @@ bool resident_available() {
 }
 
 // nsteps steps from src (time t) into dst; noise modes 0, 1 and 4
-cudaError_t launch_step_resident(const StepArgs& a, const StepArgsD& d, long long t, int nsteps, int noise_mode, int fp16,
-                                 bool poly, cudaStream_t s) {
+cudaError_t launch_step_resident(const StepArgs& a, const StepArgsD& d, long long t, int nsteps, int noise_mode, bool poly,
+                                 cudaStream_t s) {
     ResArgs r;
-    const double c = fp16 ? pair_scale<true>() : pair_scale<false>();
     const double L[4] = {d.L44, d.L49, d.L94, d.L99}, s3[3] = {d.s5, d.s6, d.s7};
-    pair_coef(d.rho0, d.cs2m, d.kappa, d.lb, d.ls, d.lq, d.le, L, s3, c, &r.c);
-    pair_local(d.e2, d.e3, d.e4, d.cq, d.lu, c, &r.loc);
+    pair_coef(d.rho0, d.cs2m, d.kappa, d.lb, d.ls, d.lq, d.le, L, s3, &r.c);
+    pair_local(d.e2, d.e3, d.e4, d.cq, d.lu, &r.loc);
     r.c.rk = a.rk;
     r.c.t_lo = r.c.t_hi = 0;
     r.g = a.g;
-    r.src = a.src;
-    r.dst = a.dst;
+    r.src = static_cast<const float*>(a.src);
+    r.dst = static_cast<float*>(a.dst);
     r.t = t;
     r.steps = nsteps;
     const int rows = (a.g.ny + RES_CTAS - 1) / RES_CTAS;
@@ -254,9 +240,12 @@ cudaError_t launch_step_resident(const StepArgs& a, const StepArgsD& d, long lon
     r.ps = r.pw * (rows + 4);
     r.nown = rows * a.g.nx / 2;
     const int threads = (r.nown + a.g.nx + 31) / 32 * 32;
-    const size_t smem = (size_t)2 * Q * r.ps * (fp16 ? 2 : 4) + (size_t)(rows + 2) * (a.g.nx + 4) * sizeof(float);
-    return fp16 ? launch_res_t<__half>(r, noise_mode, poly, threads, smem, s)
-                : launch_res_t<float>(r, noise_mode, poly, threads, smem, s);
+    const size_t smem = res_buf_bytes(r) + (size_t)(rows + 2) * (a.g.nx + 4) * sizeof(float);
+    switch (noise_mode) {
+        case 0: return poly ? launch_res<0, true>(r, threads, smem, s) : launch_res<0, false>(r, threads, smem, s);
+        case 1: return poly ? launch_res<1, true>(r, threads, smem, s) : launch_res<1, false>(r, threads, smem, s);
+        default: return poly ? launch_res<4, true>(r, threads, smem, s) : launch_res<4, false>(r, threads, smem, s);
+    }
 }
 
 }  // namespace lbf

@@ -1,9 +1,10 @@
-// lb_step_tma.cu -- the fused fluctuating D2Q9 step, TMA-staged and persistent.
+// lb_step_tma.cu -- the fused fluctuating D2Q9 step of FP32 lattices, TMA-staged and persistent (FP16
+// lattices: lb_step_half.cu).
 //
 // Same arithmetic as lb_step.cu (collide_node), two nodes at a time (collide_pair of lb_pair.cuh),
 // and different data movement:
 //   * a persistent grid (resident CTAs only) walks the lattice in TX x TY tiles (the shape
-//     chosen per noise mode and storage, tma_default_tile) in row-major tile order, so the
+//     chosen per noise mode, tma_default_tile) in row-major tile order, so the
 //     tiles in flight form a band whose halo rows are still in L2 when the neighbouring tile
 //     reads them;
 //   * for each tile one thread issues nine 3D TMA loads (cp.async.bulk.tensor), one per
@@ -26,17 +27,14 @@
 // in flight per SM and 233 us with 147 KB).
 //
 // Step at 4096^2, before and after this form (scalar nodes, two stages, stores by thread):
-// FP32 without noise 262 -> 186 us, uncorrelated 212 -> 191 (6.32 TB/s of the 72 bytes a node),
-// k-space correlated (the step kernel) 235 -> 221 less launch, real space 333 -> 263, local
-// density 219 -> 194; FP16 uncorrelated 220 -> 182, 237 instructions a node against 375.  What
-// bounds it now: FP32 DRAM; FP16 and the real-space noise the SM (FMA-heavy pipe 60 % busy, half
-// of it the wide multiplies of Philox, and the barriers between the passes).
+// without noise 262 -> 186 us, uncorrelated 212 -> 191 (6.32 TB/s of the 72 bytes a node), k-space
+// correlated (the step kernel alone) 235 -> 221, real space 333 -> 263, local density 219 -> 194.  What
+// bounds it now: DRAM; the real-space noise the SM (FMA-heavy pipe 60 % busy, half of it the wide
+// multiplies of Philox, and the barriers between the passes).
 //
 // Waits on the mbarriers are bounded by the global timer; a CTA that gives up sets the
 // error word, gives its loads in flight a bounded chance to land, and returns.
 #include <cuda.h>
-
-#include <type_traits>
 
 #include "lb_pair.cuh"
 
@@ -47,7 +45,7 @@ namespace lbf {
 struct TmaArgs : PairCoef, PairStencil {
     PairLocal loc;     // POLY and MODE 4
     Grid g;
-    void* dst;
+    float* dst;
     const float2* xi49;
     int ntx, nty;      // tiles along x and y
     int* err;          // device error word (1 = a TMA wait timed out)
@@ -56,23 +54,21 @@ struct TmaArgs : PairCoef, PairStencil {
 };
 
 // POLY: the double-well equation of state (the bulk pressure's quartic in drho)
-template <int TX, int TY, int NT, int MODE, typename T, bool POLY = false>
+template <int TX, int TY, int NT, int MODE, bool POLY = false>
 __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>()))
     step_tma_kernel(const __grid_constant__ CUtensorMap lmap, const __grid_constant__ CUtensorMap smap,
                     const TmaArgs a) {
-    using TT = TmaTile<TX, TY, T>;
+    using TT = TmaTile<TX, TY>;
     using M = PairMap<TX, TY, NT>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    T* S = reinterpret_cast<T*>(smem_raw);
-    T* out = reinterpret_cast<T*>(smem_raw + TT::OUT);
+    float* S = reinterpret_cast<float*>(smem_raw);
+    float* out = reinterpret_cast<float*>(smem_raw + TT::OUT);
     float* R = reinterpret_cast<float*>(smem_raw + TT::RHO);
     const uint32_t bar = smem_u32(smem_raw + TT::BAR);
     unsigned char* xch = smem_raw + TT::SMEM_BYTES;     // MODE 3: StencilTile
     const Grid g = a.g;
     const int tid = threadIdx.x;
     const int ntiles = a.ntx * a.nty;
-    // FP16 storage collides in the stored form g_i = df_i / w_i (no scaling on load or store)
-    constexpr bool GF = std::is_same<T, __half>::value;
 
     if (tid == 0) {
         mbar_init(bar, 1);
@@ -114,7 +110,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>())
             }
             return;
         }
-        if (tid == 0 && k > 0 && !tile_direct<TX, T>(g, px0)) {
+        if (tid == 0 && k > 0 && !tile_direct<TX>(g, px0)) {
             tma_store_3d(&smap, smem_u32(out), px0, py0, 0);
             tma_store_commit();
         }
@@ -131,7 +127,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>())
         // each thread pulls its pairs of nodes once, keeps them in registers across the barrier
         // and writes their density to the tile; the ring is formed separately
         F2 fr[M::RPT][Q];
-        tile_pull<TX, TY, NT, GF, MODE == 3>(S, R, fr);
+        tile_pull<TX, TY, NT, MODE == 3>(S, R, fr);
         F2 z4[M::RPT], z9[M::RPT];
         if constexpr (MODE == 3) stencil_tile<TX, TY, NT>(a, xch, x0, y0, g.nx, g.ny, z4, z9);
         if (tid == 0) tma_store_wait_read();
@@ -141,12 +137,11 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>())
             fence_async_smem();
             load(tcol, trow);
         }
-        tile_collide<MODE, POLY, GF, TX, TY, NT>(a, &a.loc, fr, R, g, x0, y0, out, static_cast<T*>(a.dst), a.xi49, z4,
-                                                 z9, xch);
+        tile_collide<MODE, POLY, TX, TY, NT>(a, &a.loc, fr, R, g, x0, y0, out, a.dst, a.xi49, z4, z9, xch);
         fence_async_smem();
     }
     __syncthreads();
-    if (tid == 0 && k > 0 && !tile_direct<TX, T>(g, px0)) {
+    if (tid == 0 && k > 0 && !tile_direct<TX>(g, px0)) {
         tma_store_3d(&smap, smem_u32(out), px0, py0, 0);
         tma_store_commit();
         tma_store_wait();
@@ -173,23 +168,23 @@ static const int kTiles[5][3] = {{32, 16, 256}, {32, 32, 256}, {64, 8, 256}, {64
 int tma_tile_count() { return 5; }
 
 // The fastest shape per noise mode (0 off, 1 uncorrelated, 2 correlated, 3 correlated built in real
-// space, 4 local density) and storage, measured at 4096^2 (us a step, shapes 0 to 4):
-//   FP32 off 191 208 186 205 190, uncorrelated 194 213 191 209 193, correlated (kernel alone) 232 257
-//   221 225 229, real space 294 281 304 402 263, local 195 218 194 211 198;
-//   FP16 off 140 - 134 - 133, uncorrelated 186 185 183 188 182, real space 300 - 312 - 276.
+// space, 4 local density) and storage, measured at 4096^2 (FP32, us a step, shapes 0 to 4):
+//   off 191 208 186 205 190, uncorrelated 194 213 191 209 193, correlated (kernel alone) 232 257
+//   221 225 229, real space 294 281 304 402 263, local 195 218 194 211 198.
 // Four CTAs per SM hide each other's barriers: one pair a thread where the registers allow 32 warps
 // (shape 2), two pairs and 16 warps where the contributions of the real-space noise need them
 // (shape 4: their exchange stays within a thread for half the rows).  2048^2 and 3000^2 agree; below
-// 512^2 a step is bound by its launch and the shape does not matter.
+// 512^2 a step is bound by its launch and the shape does not matter.  FP16 (lb_step_half.cu): the shapes
+// its recorded states were computed with, the fastest of that kernel.
 int tma_default_tile(int noise_mode, int fp16) {
-    static const int best[2][5] = {{2, 2, 2, 4, 2}, {4, 4, 2, 4, 2}};
+    static const int best[2][5] = {{2, 2, 2, 4, 2}, {4, 1, 3, 0, 1}};
     const int m = noise_mode < 0 ? 0 : (noise_mode > 4 ? 4 : noise_mode);
     return best[fp16 ? 1 : 0][m];
 }
 
 // Tensor maps over one population buffer.  For loads: dims (pitch, ny + 2 GY, 9), a plane's box of
-// the tile with its halo.  For stores: dims (nx, ny, 9) from node (0, 0), so that a ragged tile is
-// clipped to the lattice, the nine planes of the tile in one box.
+// the tile with its halo.  For stores (FP32): dims (nx, ny, 9) from node (0, 0), so that a ragged tile
+// is clipped to the lattice, the nine planes of the tile in one box.
 bool make_pop_tensor_maps(const void* buf, const Grid& g, int tile, int fp16, void* load_map, void* store_map) {
     EncodeTiledFn fn = tensor_map_encoder();
     if (!fn || tile < 0 || tile >= tma_tile_count()) return false;
@@ -204,6 +199,7 @@ bool make_pop_tensor_maps(const void* buf, const Grid& g, int tile, int fp16, vo
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
+    if (fp16) return true;
     cuuint64_t sdims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)Q};
     cuuint32_t sbox[3] = {(cuuint32_t)kTiles[tile][0], (cuuint32_t)kTiles[tile][1], (cuuint32_t)Q};
     return fn(reinterpret_cast<CUtensorMap*>(store_map), dt, 3, (char*)buf + g.at(0, 0) * es, sdims, strides, sbox, estr,
@@ -213,10 +209,10 @@ bool make_pop_tensor_maps(const void* buf, const Grid& g, int tile, int fp16, vo
 
 size_t tensor_map_bytes() { return sizeof(CUtensorMap); }
 
-template <int TX, int TY, int NT, int MODE, typename T, bool POLY = false>
+template <int TX, int TY, int NT, int MODE, bool POLY = false>
 static cudaError_t launch_cfg(const void* const map[2], TmaArgs ta, cudaStream_t s) {
-    using TT = TmaTile<TX, TY, T>;
-    auto kern = step_tma_kernel<TX, TY, NT, MODE, T, POLY>;
+    using TT = TmaTile<TX, TY>;
+    auto kern = step_tma_kernel<TX, TY, NT, MODE, POLY>;
     constexpr int smem = TT::SMEM_BYTES + (MODE == 3 ? StencilTile<TX, TY, NT>::BYTES : 0);
     static GridCache cache;
     int grid_max = 0;
@@ -230,25 +226,14 @@ static cudaError_t launch_cfg(const void* const map[2], TmaArgs ta, cudaStream_t
                           *static_cast<const CUtensorMap*>(map[1]), ta);
 }
 
-template <int MODE, typename T>
+template <int MODE>
 static cudaError_t launch_mode(const void* const map[2], const TmaArgs& ta, int tile, cudaStream_t s) {
     switch (tile) {
-        case 1: return launch_cfg<32, 32, 256, MODE, T>(map, ta, s);
-        case 2: return launch_cfg<64, 8, 256, MODE, T>(map, ta, s);
-        case 3: return launch_cfg<64, 16, 512, MODE, T>(map, ta, s);
-        case 4: return launch_cfg<32, 16, 128, MODE, T>(map, ta, s);
-        default: return launch_cfg<32, 16, 256, MODE, T>(map, ta, s);
-    }
-}
-
-template <typename T>
-static cudaError_t launch_type(const void* const map[2], const TmaArgs& ta, int noise_mode, int tile, cudaStream_t s) {
-    switch (noise_mode) {
-        case 0: return launch_mode<0, T>(map, ta, tile, s);
-        case 1: return launch_mode<1, T>(map, ta, tile, s);
-        case 3: return launch_mode<3, T>(map, ta, tile, s);
-        case 4: return launch_mode<4, T>(map, ta, tile, s);
-        default: return launch_mode<2, T>(map, ta, tile, s);
+        case 1: return launch_cfg<32, 32, 256, MODE>(map, ta, s);
+        case 2: return launch_cfg<64, 8, 256, MODE>(map, ta, s);
+        case 3: return launch_cfg<64, 16, 512, MODE>(map, ta, s);
+        case 4: return launch_cfg<32, 16, 128, MODE>(map, ta, s);
+        default: return launch_cfg<32, 16, 256, MODE>(map, ta, s);
     }
 }
 
@@ -256,25 +241,24 @@ static cudaError_t launch_type(const void* const map[2], const TmaArgs& ta, int 
 // (tma_default_tile(noise_mode, 0); the caller encodes the tensor maps for it)
 static cudaError_t launch_poly(const void* const map[2], const TmaArgs& ta, int noise_mode, cudaStream_t s) {
     switch (noise_mode) {
-        case 0: return launch_cfg<64, 8, 256, 0, float, true>(map, ta, s);
-        case 1: return launch_cfg<64, 8, 256, 1, float, true>(map, ta, s);
-        case 3: return launch_cfg<32, 16, 128, 3, float, true>(map, ta, s);
-        case 4: return launch_cfg<64, 8, 256, 4, float, true>(map, ta, s);
-        default: return launch_cfg<64, 8, 256, 2, float, true>(map, ta, s);
+        case 0: return launch_cfg<64, 8, 256, 0, true>(map, ta, s);
+        case 1: return launch_cfg<64, 8, 256, 1, true>(map, ta, s);
+        case 3: return launch_cfg<32, 16, 128, 3, true>(map, ta, s);
+        case 4: return launch_cfg<64, 8, 256, 4, true>(map, ta, s);
+        default: return launch_cfg<64, 8, 256, 2, true>(map, ta, s);
     }
 }
 
-cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* src_map, const void* dst_map, int* err, int noise_mode, int tile, int fp16,
+cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* src_map, const void* dst_map, int* err, int noise_mode, int tile,
                             cudaStream_t s, bool poly) {
     TmaArgs ta;
-    const double c = fp16 ? pair_scale<true>() : pair_scale<false>();
     // the coefficients from FP64, rounded once
     const double L[4] = {d.L44, d.L49, d.L94, d.L99}, s3[3] = {d.s5, d.s6, d.s7};
-    pair_coef(d.rho0, d.cs2m, d.kappa, d.lb, d.ls, d.lq, d.le, L, s3, c, &ta);
-    pair_stencil(d.sL, c, &ta);
-    pair_local(d.e2, d.e3, d.e4, d.cq, d.lu, c, &ta.loc);
+    pair_coef(d.rho0, d.cs2m, d.kappa, d.lb, d.ls, d.lq, d.le, L, s3, &ta);
+    pair_stencil(d.sL, &ta);
+    pair_local(d.e2, d.e3, d.e4, d.cq, d.lu, &ta.loc);
     ta.g = a.g;
-    ta.dst = a.dst;
+    ta.dst = static_cast<float*>(a.dst);
     ta.xi49 = a.xi49;
     ta.ntx = ta.nty = 0;
     ta.err = err;
@@ -282,9 +266,14 @@ cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* s
     ta.t_hi = a.t_hi;
     ta.rk = a.rk;
     const void* const map[2] = {src_map, dst_map};
-    if (poly) return fp16 ? cudaErrorInvalidValue : launch_poly(map, ta, noise_mode, s);
-    return fp16 ? launch_type<__half>(map, ta, noise_mode, tile, s)
-                : launch_type<float>(map, ta, noise_mode, tile, s);
+    if (poly) return launch_poly(map, ta, noise_mode, s);
+    switch (noise_mode) {
+        case 0: return launch_mode<0>(map, ta, tile, s);
+        case 1: return launch_mode<1>(map, ta, tile, s);
+        case 3: return launch_mode<3>(map, ta, tile, s);
+        case 4: return launch_mode<4>(map, ta, tile, s);
+        default: return launch_mode<2>(map, ta, tile, s);
+    }
 }
 
 }  // namespace lbf

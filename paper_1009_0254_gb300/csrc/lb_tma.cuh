@@ -7,20 +7,20 @@
 
 namespace lbf {
 
-// Shared memory of one CTA that steps TX x TY tiles: the stage (nine boxes of the tile being
+// Shared memory of one CTA that steps TX x TY tiles of an FP32 lattice: the stage (nine boxes of the tile being
 // loaded or pulled), the nine post-collision planes on their way out, the density tile with its
 // one-node ring, and the mbarrier.
-template <int TX, int TY, typename T>
+template <int TX, int TY>
 struct TmaTile {
-    static constexpr int XO = Elem<T>::XO;                              // 16 bytes of elements
+    static constexpr int XO = Elem<float>::XO;                              // 16 bytes of elements
     static constexpr int BW = TX + 2 * XO;                              // box width (elements)
     static constexpr int BH = TY + 2;                                   // box height
-    static constexpr int PLANE_BYTES = BW * BH * (int)sizeof(T);
-    static constexpr int PS = ((PLANE_BYTES + 127) / 128) * 128 / (int)sizeof(T);   // plane stride (elements)
-    static constexpr int STAGE_BYTES = Q * PS * (int)sizeof(T);
+    static constexpr int PLANE_BYTES = BW * BH * (int)sizeof(float);
+    static constexpr int PS = ((PLANE_BYTES + 127) / 128) * 128 / (int)sizeof(float);   // plane stride (elements)
+    static constexpr int STAGE_BYTES = Q * PS * (int)sizeof(float);
     static constexpr uint32_t TX_BYTES = Q * PLANE_BYTES;
     static constexpr int OUT = STAGE_BYTES;                             // [plane][TY][TX]: one box of the store map
-    static constexpr int OUT_BYTES = Q * TX * TY * (int)sizeof(T);
+    static constexpr int OUT_BYTES = Q * TX * TY * (int)sizeof(float);
     static_assert(OUT % 128 == 0 && OUT_BYTES % 128 == 0, "boxes start on 128 bytes");
     // density tile + ring, node (lx, ly) at (ly + 1) RW + lx + 2: pairs of columns (lx even) on
     // 8-byte boundaries
