@@ -202,8 +202,8 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
         fence_async_smem();
     }
     __syncthreads();
-    if (tid == 0 && k > 0) {
-        store(pos[(k - 1u) & 1u]);
+    if (tid == 0) {
+        if (k > 0) store(pos[(k - 1u) & 1u]);
         tma_store_wait();
     }
     // Every CTA read K before arriving here; the last one to arrive advances it for the

@@ -214,8 +214,8 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
         fence_async_smem();
     }
     __syncthreads();
-    if (tid == 0 && k > 0) {
-        store((int)((k - 1u) & 1u));
+    if (tid == 0) {
+        if (k > 0) store((int)((k - 1u) & 1u));
         tma_store_wait();
     }
     if (tid == 0) {

@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>())
                 // give the loads still in flight into this CTA's shared memory a bounded
                 // chance to land before the CTA exits
                 mbar_wait_bounded(bar, k & 1u);
+                tma_store_wait();
             }
             return;
         }
@@ -141,10 +142,12 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, MODE == 3>())
         fence_async_smem();
     }
     __syncthreads();
-    if (tid == 0 && k > 0 && !tile_direct<TX>(g, px0)) {
-        tma_store_3d(&smap, smem_u32(out), px0, py0, 0);
-        tma_store_commit();
-        tma_store_wait();
+    if (tid == 0 && k > 0) {
+        if (!tile_direct<TX>(g, px0)) {
+            tma_store_3d(&smap, smem_u32(out), px0, py0, 0);
+            tma_store_commit();
+        }
+        tma_store_wait();              // of earlier tiles too, if the last one left by its threads
     }
 }
 
