@@ -23,6 +23,7 @@
 
 #include "lb_ens.cuh"
 #include "lb_fft_core.cuh"
+#include "lb_limits.cuh"
 #include "lb_noise.cuh"
 #include "lb_spectra.cuh"
 #include "lbfluct.h"
@@ -813,7 +814,6 @@ int lb_batch_create(int count, const int* nx, const int* ny, const uint64_t* see
     }
     cudaError_t e = cudaMemset(b->ws, 0, b->L.total);
     std::vector<float2> tw;
-    size_t noise_csm = 0, noise_rsm = 0;
     for (auto& ci : b->L.classes) {
         if (e != cudaSuccess) break;
         for (int which = 0; which < 2; ++which) {
@@ -831,12 +831,6 @@ int lb_batch_create(int count, const int* nx, const int* ny, const uint64_t* see
             e = cudaMemcpy(cls_ptr(b, which == 0 ? ci.off_cosx : ci.off_cosy), cs.data(), n * sizeof(float),
                            cudaMemcpyHostToDevice);
         }
-        if (e == cudaSuccess && pow2b(ci.nx) && pow2b(ci.ny) && ci.ny <= 8192) {
-            // shared memory of the correlated-noise kernels, set before any graph capture
-            const int c = col_strip_b(ci.nx, ci.ny);
-            noise_csm = std::max(noise_csm, fft_smem_bytes(ci.ny, c));
-            noise_rsm = std::max(noise_rsm, fft_smem_bytes(ci.nx, noise_rows_per_cta(ci.nx, ci.ny)));
-        }
     }
     for (int r = 0; r < count && e == cudaSuccess; ++r) {
         const ClassInfo& ci = b->L.classes[b->L.cls_of[r]];
@@ -845,10 +839,9 @@ int lb_batch_create(int count, const int* nx, const int* ny, const uint64_t* see
     }
     if (e == cudaSuccess) e = cudaMemcpy(cls_ptr(b, b->L.off_fbar), b->fbar, sizeof(double) * Q, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = prepare_ensemble_kernels();
-    if (e == cudaSuccess && noise_csm > 0)
-        e = cudaFuncSetAttribute(batch_noise_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)noise_csm);
-    if (e == cudaSuccess && noise_rsm > 0)
-        e = cudaFuncSetAttribute(batch_noise_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)noise_rsm);
+    // shared memory of the correlated-noise kernels, raised before any graph capture
+    if (e == cudaSuccess) e = all_shared_memory<batch_noise_cols_kernel>();
+    if (e == cudaSuccess) e = all_shared_memory<batch_noise_rows_kernel>();
     {
         // LBFLUCT_BATCH_TILE=<0..6> fixes the tile shape until an autotune (tests of every shape)
         const char* tv = std::getenv("LBFLUCT_BATCH_TILE");
@@ -1122,17 +1115,12 @@ int lb_batch_set_sampling(lb_batch* b, int every, int nbins) {
     if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; b->graph_steps = 0; }
     if (every == 0) { b->every = 0; return LB_OK; }
     if (nbins < 1 || nbins > kMaxBatchBins) return bfail(b, LB_EINVAL, "nbins must lie in [1, 1024]");
-    size_t rsm = 0, csm = 0;
-    for (auto& ci : b->L.classes) {
+    for (auto& ci : b->L.classes)
         if (!pow2b(ci.nx) || !pow2b(ci.ny)) return bfail(b, LB_EINVAL, "spectra need power-of-two lattice sides");
-        rsm = std::max(rsm, fft_smem_bytes(ci.nx, 1));
-        csm = std::max(csm, fft_smem_bytes(ci.ny, col_strip_b(ci.nx, ci.ny)));
-    }
-    // shared memory of the sample kernels, set here so that a graph capture makes no such call
-    BCK(b, cudaFuncSetAttribute(batch_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm), "attr");
-    BCK(b, cudaFuncSetAttribute(batch_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm), "attr");
-    BCK(b, cudaFuncSetAttribute(batch_bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(3 * nbins * sizeof(double))), "attr");
+    // shared memory of the sample kernels, raised here so that a graph capture makes no such call
+    BCK(b, all_shared_memory<batch_rows_kernel>(), "attr");
+    BCK(b, all_shared_memory<batch_cols_kernel>(), "attr");
+    BCK(b, all_shared_memory<batch_bin_kernel>(), "attr");
     b->every = every;
     b->nbins = nbins;
     b->nsamples = 0;

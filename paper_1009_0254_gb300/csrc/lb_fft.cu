@@ -14,6 +14,7 @@
 
 #include "lb_fft_core.cuh"
 #include "lb_internal.cuh"
+#include "lb_limits.cuh"
 #include "lb_noise.cuh"
 #include "lb_spectra.cuh"
 
@@ -131,27 +132,23 @@ static int noise_strip(int nx, int c) {
     return c;
 }
 
-// launch of a transform kernel (its dynamic shared-memory limit raised where it asks for more than
-// the 48 KB that every kernel may use)
-template <typename... P, typename... A>
-static cudaError_t launch_fft(void (*kern)(P...), int grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    return launch_chained(kern, dim3(grid), dim3(threads), smem, s, std::forward<A>(args)...);
+// launch of a transform kernel, for which sizes that need more shared memory than a CTA has are refused
+template <auto Kern, typename... A>
+static cudaError_t launch_fft(int grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+    const cudaError_t e = all_shared_memory<Kern>();
+    return e != cudaSuccess ? e : launch_chained(Kern, dim3(grid), dim3(threads), smem, s, std::forward<A>(args)...);
 }
 
 static cudaError_t rows_pass(float2* data, int nx, int ny, int sign, const float2* twx, float scale,
                              cudaStream_t s) {
-    return launch_fft(fft_rows_kernel, ny, fft_threads(nx, 1), fft_smem_bytes(nx, 1), s, data, nx, sign, twx, scale);
+    return launch_fft<fft_rows_kernel>(ny, fft_threads(nx, 1), fft_smem_bytes(nx, 1), s, data, nx, sign, twx, scale);
 }
 
 static cudaError_t cols_pass(float2* data, int nx, int ny, int sign, const float2* twy, float scale,
                              cudaStream_t s) {
     const int c = col_strip(nx, ny);
-    return launch_fft(fft_cols_kernel, nx / c, fft_threads(ny, c), fft_smem_bytes(ny, c), s, data, nx, ny, c, sign, twy,
-                      scale);
+    return launch_fft<fft_cols_kernel>(nx / c, fft_threads(ny, c), fft_smem_bytes(ny, c), s, data, nx, ny, c, sign, twy,
+                                       scale);
 }
 
 cudaError_t launch_fft2d(float2* data, int nx, int ny, int sign, const float2* twx, const float2* twy,
@@ -174,13 +171,13 @@ cudaError_t launch_noise49(float2* buf, float2* scratch, const NoiseGenArgs& ga,
     const float scale = (float)(1.0 / sqrt((double)ga.nx * (double)ga.ny));
     cudaError_t e;
     if (ga.nx < 256) {
-        e = launch_fft(noise_cols_kernel<false>, ga.nx / c, fft_threads(ga.ny, c), smem, s, buf, ga, c, twy);
+        e = launch_fft<noise_cols_kernel<false>>(ga.nx / c, fft_threads(ga.ny, c), smem, s, buf, ga, c, twy);
         return e != cudaSuccess ? e : rows_pass(buf, ga.nx, ga.ny, -1, twx, scale, s);
     }
-    e = launch_fft(noise_cols_kernel<true>, ga.nx / c, fft_threads(ga.ny, c), smem, s, scratch, ga, c, twy);
+    e = launch_fft<noise_cols_kernel<true>>(ga.nx / c, fft_threads(ga.ny, c), smem, s, scratch, ga, c, twy);
     if (e != cudaSuccess) return e;
-    return launch_fft(noise_rows_kernel, ga.ny, fft_threads(ga.nx, 1), fft_smem_bytes(ga.nx, 1), s, scratch, buf, ga.nx,
-                      ga.ny, c, twx, scale);
+    return launch_fft<noise_rows_kernel>(ga.ny, fft_threads(ga.nx, 1), fft_smem_bytes(ga.nx, 1), s, scratch, buf, ga.nx,
+                                         ga.ny, c, twx, scale);
 }
 
 int noise_strip_d(int nx, int ny) {
@@ -195,11 +192,11 @@ cudaError_t launch_noise49_d(double2* buf, const NoiseGenArgsD& ga, const double
     if (c < 2) return cudaErrorInvalidValue;
     // a thread per radix-4 butterfly or per pair of wavevectors, whichever is more (both at most 512)
     auto threads = [](int n) { return n < 32 ? 32 : (n > 512 ? 512 : n); };
-    const cudaError_t e = launch_fft(noise_cols_kernel_d, ga.nx / c, threads(ga.ny * c / 2), fft_smem_bytes(ga.ny, c, 16), s,
-                                     buf, ga, c, twy);
+    const cudaError_t e = launch_fft<noise_cols_kernel_d>(ga.nx / c, threads(ga.ny * c / 2),
+                                                          fft_smem_bytes(ga.ny, c, 16), s, buf, ga, c, twy);
     if (e != cudaSuccess) return e;
-    return launch_fft(fft_rows_kernel_d, ga.ny, threads(ga.nx / 4), fft_smem_bytes(ga.nx, 1, 16), s, buf, ga.nx, -1, twx,
-                      1.0 / sqrt((double)ga.nx * (double)ga.ny));
+    return launch_fft<fft_rows_kernel_d>(ga.ny, threads(ga.nx / 4), fft_smem_bytes(ga.nx, 1, 16), s, buf, ga.nx, -1, twx,
+                                         1.0 / sqrt((double)ga.nx * (double)ga.ny));
 }
 
 // --- sampled spectra ---------------------------------------------------------------
@@ -295,8 +292,7 @@ cudaError_t launch_stats_sample(const void* pops, int storage, const Grid& g, fl
     e = launch_fft2d(z2, g.nx, g.ny, +1, twx, twy, scale, s);
     if (e != cudaSuccess) return e;
     const size_t smem = (size_t)3 * nbins * sizeof(double);
-    e = cudaFuncSetAttribute(bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if ((e = all_shared_memory<bin_kernel>()) != cudaSuccess) return e;
     const long long units = (long long)(g.ny / 2 + 1) * ((g.nx / 2 + 32) / 32);   // warp work units
     // two CTAs per SM, of 16 warps where there are four units for each (a warp's loads of a unit are one
     // latency: 4096^2 a sample 619 us with 8 warps, 554 with 16; 2048^2 155, 144), of 8 below (256^2 37.6

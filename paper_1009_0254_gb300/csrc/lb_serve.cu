@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "lb_ens.cuh"
+#include "lb_limits.cuh"
 #include "lb_noise.cuh"
 #include "lbfluct.h"
 
@@ -380,7 +381,6 @@ struct lb_server {
     int* d_full[2] = {nullptr, nullptr};     // correlated simulations of a chunk, grouped by size
     int* h_full[2] = {nullptr, nullptr};
     std::map<std::pair<int, int>, SizeTables> tables;
-    size_t noise_csm = 0, noise_rsm = 0;     // shared memory the noise kernels are set up for
     int* d_tb[2] = {nullptr, nullptr};
     int4* d_tiles = nullptr;                 // tile records of the current chunk (grown on demand)
     int tiles_cap = 0;
@@ -464,15 +464,8 @@ bool ensure_tables(lb_server* s, int nx, int ny) {
         SCK(s, cudaMemcpy(which == 0 ? t.cosx : t.cosy, cs.data(), n * sizeof(float), cudaMemcpyHostToDevice));
     }
     s->tables[key] = t;
-    const size_t csm = fft_smem_bytes(ny, noise_strip(nx, ny)), rsm = fft_smem_bytes(nx, 1);
-    if (csm > s->noise_csm) {
-        SCK(s, cudaFuncSetAttribute(serve_noise_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
-        s->noise_csm = csm;
-    }
-    if (rsm > s->noise_rsm) {
-        SCK(s, cudaFuncSetAttribute(serve_noise_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
-        s->noise_rsm = rsm;
-    }
+    SCK(s, all_shared_memory<serve_noise_cols_kernel>());
+    SCK(s, all_shared_memory<serve_noise_rows_kernel>());
     return true;
 }
 

@@ -16,6 +16,7 @@
 
 #include <atomic>
 
+#include "lb_limits.cuh"
 #include "lb_pair.cuh"
 
 namespace lbf {
@@ -171,9 +172,9 @@ bool resident_fits(const Grid& g) {
 
 template <int MODE, bool POLY>
 static cudaError_t launch_res(const ResArgs& a, int threads, size_t smem, cudaStream_t s) {
-    auto kern = step_resident_kernel<MODE, POLY>;
+    constexpr auto kern = step_resident_kernel<MODE, POLY>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = all_shared_memory<kern>();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t c = {};
     c.gridDim = dim3(RES_CTAS);
@@ -198,7 +199,7 @@ bool resident_available() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return false;
     int k = known[dev].load(std::memory_order_acquire);
     if (k == 0) {
-        auto kern = step_resident_kernel<1, false>;
+        constexpr auto kern = step_resident_kernel<1, false>;
         const int smem = 2 * Q * (RES_MAX_NX + 8) * 12 * 4 + 10 * (RES_MAX_NX + 4) * 4;
         cudaLaunchConfig_t c = {};
         c.gridDim = dim3(RES_CTAS);
@@ -212,7 +213,7 @@ bool resident_available() {
         c.numAttrs = 1;
         int n = 0;
         const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                        all_shared_memory<kern>() == cudaSuccess &&
                         cudaOccupancyMaxActiveClusters(&n, kern, &c) == cudaSuccess && n > 0;
         if (!ok) cudaGetLastError();
         k = ok ? 1 : 2;
