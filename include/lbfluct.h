@@ -349,7 +349,8 @@ const char* lb_batch_last_error(lb_batch* b);
  *   LB_NOISE_FULL); 0 for an invalid size (sides in [2, 16384]).
  * lb_server_create: starts a scheduler thread on the current device.  hbm_budget_bytes
  *   bounds the sum of lb_server_request_bytes over admitted requests (their memory comes
- *   from a stream-ordered pool that keeps up to the budget cached); max_active bounds the
+ *   from a stream-ordered pool that keeps up to the budget cached, as do 16 bytes per 512
+ *   nodes of records that the budget does not count); max_active bounds the
  *   number admitted at once (device tables are sized for it); max_chunk_steps bounds the
  *   steps issued between two admission decisions.  Requests are admitted in arrival order;
  *   one that does not fit the remaining budget lets later, smaller ones pass.

@@ -382,7 +382,7 @@ struct lb_server {
     int* h_full[2] = {nullptr, nullptr};
     std::map<std::pair<int, int>, SizeTables> tables;
     int* d_tb[2] = {nullptr, nullptr};
-    int4* d_tiles = nullptr;                 // tile records of the current chunk (grown on demand)
+    int4* d_tiles = nullptr;                 // tile records of the current chunk (reserve_tiles)
     int tiles_cap = 0;
     long long* d_k = nullptr;
     unsigned int* d_done = nullptr;
@@ -521,6 +521,25 @@ bool apply_cancellations(lb_server* s) {
     return true;
 }
 
+int grid_tiles(const Grid& g) { return ((g.nx + SV_TX - 1) / SV_TX) * ((g.ny + SV_TY - 1) / SV_TY); }
+
+// room for the tile records of the running simulations and one more of grid g (16 bytes per 512 nodes);
+// the table in use is kept if there is no memory for a larger one
+cudaError_t reserve_tiles(lb_server* s, const Grid& g) {
+    int tiles = grid_tiles(g);
+    for (const Running& r : s->running) tiles += grid_tiles(r.g);
+    if (tiles <= s->tiles_cap) return cudaSuccess;
+    const int cap = std::max(4096, tiles + tiles / 2);
+    void* table = nullptr;
+    cudaError_t e = cudaMallocFromPoolAsync(&table, (size_t)cap * sizeof(int4), s->pool, s->stream);
+    if (e != cudaSuccess) return e;
+    // the chunks issued so far are ahead in the stream, and each chunk writes its own records
+    if (s->d_tiles) e = cudaFreeAsync(s->d_tiles, s->stream);
+    s->d_tiles = static_cast<int4*>(table);
+    s->tiles_cap = cap;
+    return e;
+}
+
 // admit pending requests (arrival order, smaller ones may pass a request that does not fit)
 bool admit(lb_server* s) {
     std::vector<Pending> take;
@@ -578,8 +597,10 @@ bool admit(lb_server* s) {
         void* mem = nullptr;
         cudaError_t ae = injected ? cudaErrorMemoryAllocation
                                   : cudaMallocFromPoolAsync(&mem, run.bytes, s->pool, s->stream);
+        if (ae == cudaSuccess) ae = reserve_tiles(s, run.g);
         if (ae == cudaErrorMemoryAllocation) {
             cudaGetLastError();            // not sticky: clear it
+            if (mem) SCK(s, cudaFreeAsync(mem, s->stream));
             finish_unrun(s, run, LB_ENOMEM);
             continue;
         }
@@ -714,7 +735,7 @@ bool issue_chunk(lb_server* s) {
         const Running& r = s->running[a];
         act[a] = r.slot;
         tb[a] = tiles;
-        tiles += ((r.g.nx + SV_TX - 1) / SV_TX) * ((r.g.ny + SV_TY - 1) / SV_TY);
+        tiles += grid_tiles(r.g);
         nodes += (double)r.g.nx * r.g.ny;
     }
     const int n = (int)s->running.size();
@@ -751,16 +772,7 @@ bool issue_chunk(lb_server* s) {
     p.kstep = s->d_k;
     p.done = s->d_done;
     p.err = s->d_err;
-    if (tiles > s->tiles_cap) {
-        // 16 bytes per 512 nodes; earlier chunks' launches are ahead in the stream
-        if (s->d_tiles) SCK(s, cudaFreeAsync(s->d_tiles, s->stream));
-        s->d_tiles = nullptr;
-        s->tiles_cap = 0;
-        const int cap = std::max(4096, tiles + tiles / 2);
-        SCK(s, cudaMallocFromPoolAsync((void**)&s->d_tiles, (size_t)cap * sizeof(int4), s->pool, s->stream));
-        s->tiles_cap = cap;
-    }
-    p.tiles = s->d_tiles;
+    p.tiles = s->d_tiles;              // reserve_tiles made room for them
     serve_tiles_kernel<<<(tiles + 255) / 256, 256, 0, s->stream>>>(p, SV_TX, SV_TY);
     bool rs = false;
     for (const Running& r : s->running) rs = rs || (r.r.noise_mode == LB_NOISE_FULL_RS && r.r.kT > 0.0);
