@@ -1,4 +1,5 @@
-// lb_limits.cuh -- the dynamic shared-memory limit of kernels whose launches ask for differing amounts.
+// lb_limits.cuh -- what the current device has: the dynamic shared-memory limit of kernels whose launches ask
+// for differing amounts, and the number of SMs.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -27,6 +28,19 @@ cudaError_t all_shared_memory() {
     e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
     if (e == cudaSuccess) done[dev].store(true, std::memory_order_release);
     return e;
+}
+
+// SMs of the current device, asked once (1 if it cannot be asked)
+inline int device_sms() {
+    static std::atomic<int> known[MAX_DEVICES];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return 1;
+    n = known[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+        known[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
 }
 
 }  // namespace lbf

@@ -16,6 +16,7 @@
 // small fluctuations (~sqrt(kT)) at full relative precision; with FP64 storage the
 // arithmetic is FP64 too (this kernel is the FP64 path).
 #include "lb_collide.cuh"
+#include "lb_limits.cuh"
 
 namespace lbf {
 
@@ -170,10 +171,10 @@ cudaError_t launch_step_simple(const StepArgs& a, int noise_mode, int fp16, cuda
 // the busiest SM is taken, the density ring and, with the real-space noise, the halo's draws counted.
 // Uncorrelated noise, us a step, 32 x 16 tiles alone and by this rule: 64^2 56 and 16, 512^2 212 and 188.
 cudaError_t launch_step_simple_d(const StepArgsD& a, int noise_mode, cudaStream_t s) {
-    const long long tx = (a.g.nx + 31) / 32;
+    const long long tx = (a.g.nx + 31) / 32, sms = device_sms();
     const int pairs = noise_mode == 0 ? 0 : (noise_mode == 2 ? 2 : (noise_mode == 3 ? 6 : 3));
     auto work = [&](int by) {
-        const long long ctas = tx * ((a.g.ny + by - 1) / by), turns = (ctas + 151) / 152;
+        const long long ctas = tx * ((a.g.ny + by - 1) / by), turns = (ctas + sms - 1) / sms;
         return turns * (32 * by * (150 + 115 * pairs) + (68 + 2 * by) * 8 + (noise_mode == 3 ? (33 + by) * 4 * 115 : 0));
     };
     const long long w16 = work(16), w4 = work(4), w1 = work(1);
