@@ -168,14 +168,15 @@ cudaError_t launch_step_simple(const StepArgs& a, int noise_mode, int fp16, cuda
 // FP64: an SM issues two FP64 operations a clock, and a node needs some 150 of them, plus 115 for each
 // of its Box-Muller pairs (logarithm, root, sine and cosine), so a 32 x 16 tile takes its SM 46 us and
 // what counts is that every SM has its share.  The tile height (16, 4 or 1 rows) of the least work on
-// the busiest SM is taken, the density ring and, with the real-space noise, the halo's draws counted.
+// the busiest SM is taken, the density ring and, with the real-space noise, the halo's draws (in whole
+// warps) counted.
 // Uncorrelated noise, us a step, 32 x 16 tiles alone and by this rule: 64^2 56 and 16, 512^2 212 and 188.
 cudaError_t launch_step_simple_d(const StepArgsD& a, int noise_mode, cudaStream_t s) {
     const long long tx = (a.g.nx + 31) / 32, sms = device_sms();
     const int pairs = noise_mode == 0 ? 0 : (noise_mode == 2 ? 2 : (noise_mode == 3 ? 6 : 3));
     auto work = [&](int by) {
         const long long ctas = tx * ((a.g.ny + by - 1) / by), turns = (ctas + sms - 1) / sms;
-        return turns * (32 * by * (150 + 115 * pairs) + (68 + 2 * by) * 8 + (noise_mode == 3 ? (33 + by) * 4 * 115 : 0));
+        return turns * (32 * by * (150 + 115 * pairs) + (68 + 2 * by) * 8 + (noise_mode == 3 ? (33 + by + 31) / 32 * 32 * 4 * 115 : 0));
     };
     const long long w16 = work(16), w4 = work(4), w1 = work(1);
     if (w16 <= w4 && w16 <= w1) return launch_t<double, 32, 16>(a, noise_mode, s);
