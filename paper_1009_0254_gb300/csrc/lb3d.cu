@@ -334,8 +334,9 @@ __global__ void get_plane3_kernel(const R* __restrict__ src, double* __restrict_
 
 // All populations in one launch, dst[i][z][y][x], from the ghosts where r - c_i leaves the lattice in x
 // or y: a block takes GET_ROWS rows of one plane, columns consecutive, no division (the kernel above
-// divides two 64-bit indexes per element) and no FP64 conversion (widen).  Blocks follow the populations
-// in order: a thread that wrote every population of its node would spread the stores over 19 or 27 distant
+// divides two 64-bit indexes per element) and no FP64 conversion (widen).  Narrow lattices take several runs
+// of rows a block, so that its warps are full (2 x 256 x 256 D3Q19 FP32: 151 us with one, 133 by divisions,
+// 39 this way).  Blocks follow the populations in order: a thread that wrote every population of its node would spread the stores over 19 or 27 distant
 // planes, and took as long as the divisions.  256^3 FP32, us, a launch per population with divisions,
 // without them in one launch, with widen too: D3Q19 1,468, 1,210, 842; D3Q27 2,060, 1,700, 1,191
 // (4.5 TB/s; the FP64 additions of the rest values bound it).
@@ -353,7 +354,8 @@ __global__ void get_all3_kernel(const R* __restrict__ src, double* __restrict__ 
         const R* s = src + LAT::sigma(i) * g.P + g.at(x - LAT::c(i, 0), -LAT::c(i, 1), wrap1(z - LAT::c(i, 2), g.nz));
         double* d = dst + (long long)p * g.ny * g.nx + x;
         const double f = rest.f[i];
-        for (int y0 = blockIdx.y * GET_ROWS; y0 < g.ny; y0 += gridDim.y * GET_ROWS)
+        for (int y0 = (blockIdx.y * blockDim.y + threadIdx.y) * GET_ROWS; y0 < g.ny;
+             y0 += gridDim.y * blockDim.y * GET_ROWS)
 #pragma unroll
             for (int k = 0; k < GET_ROWS; ++k)
                 if (y0 + k < g.ny) d[(long long)(y0 + k) * g.nx] = lbf::widen(s[(long long)(y0 + k) * g.pitch]) + f;
@@ -364,10 +366,12 @@ template <typename LAT, typename R>
 static cudaError_t launch_get_all3(const void* pops, double* dst, const Geom3& g, const double* fbar, cudaStream_t s) {
     Rest27 r{};
     for (int i = 0; i < LAT::Q; ++i) r.f[i] = fbar[i];
-    const int bx = g.nx > 64 ? 128 : (g.nx > 32 ? 64 : 32);
-    const dim3 grd((g.nx + bx - 1) / bx, std::min((g.ny + GET_ROWS - 1) / GET_ROWS, 65535),
-                   std::min((long long)LAT::Q * g.nz, 65535LL));
-    get_all3_kernel<LAT, R><<<grd, bx, 0, s>>>((const R*)pops, dst, g, r);
+    int bx = 128;
+    while (bx > 1 && bx / 2 >= g.nx) bx /= 2;
+    const int by = 128 / bx, rows = by * GET_ROWS;
+    const dim3 blk(bx, by), grd((g.nx + bx - 1) / bx, std::min((g.ny + rows - 1) / rows, 65535),
+                                std::min((long long)LAT::Q * g.nz, 65535LL));
+    get_all3_kernel<LAT, R><<<grd, blk, 0, s>>>((const R*)pops, dst, g, r);
     return cudaGetLastError();
 }
 
