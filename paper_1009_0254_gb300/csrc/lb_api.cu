@@ -383,7 +383,7 @@ int lb_create(int nx, int ny, int precision, uint64_t seed, double rho0, double 
         c->use_resident = !v && !tv && precision == LB_FP32 && resident_fits(g) && resident_available();
         c->tma_tile_fixed = tv ? std::atoi(tv) : -1;
         if (c->tma_tile_fixed >= tma_tile_count()) c->tma_tile_fixed = -1;
-        c->tma_tile = c->tma_tile_fixed >= 0 ? c->tma_tile_fixed : tma_default_tile(LB_NOISE_LW, c->fp16);
+        c->tma_tile = c->tma_tile_fixed >= 0 ? c->tma_tile_fixed : tma_default_tile(LB_NOISE_LW, c->fp16, g);
         c->use_tma = want_tma && tensor_map_bytes() <= sizeof(c->tmap[0]) &&
                      make_pop_tensor_maps(c->pop[0], g, c->tma_tile, c->fp16, c->tmap[0], c->tmap_out[0]) &&
                      make_pop_tensor_maps(c->pop[1], g, c->tma_tile, c->fp16, c->tmap[1], c->tmap_out[1]);
@@ -747,7 +747,7 @@ int lb_step(lb_ctx* c, int64_t nsteps) {
         if (c->use_sweep && kmode < 3 && !poly)
             CK(c, launch_step_sweep(a, kmode, c->fp16, c->sweep_occ6, c->stream), "step kernel launch");
         else if (c->use_tma && (!poly || !c->fp16)) {
-            const int want = (c->tma_tile_fixed >= 0 && !poly) ? c->tma_tile_fixed : tma_default_tile(kmode, c->fp16);
+            const int want = (c->tma_tile_fixed >= 0 && !poly) ? c->tma_tile_fixed : tma_default_tile(kmode, c->fp16, c->g);
             if (want != c->tma_tile) {
                 // tensor maps are host-encoded descriptors passed by value: re-encode for the shape
                 if (!make_pop_tensor_maps(c->pop[0], c->g, want, c->fp16, c->tmap[0], c->tmap_out[0]) ||

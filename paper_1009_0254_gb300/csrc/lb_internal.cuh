@@ -463,7 +463,7 @@ cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* s
 cudaError_t launch_step_half(const StepArgs& a, const void* src_map, int* err, int noise_mode, int tile, cudaStream_t s);
 bool make_pop_tensor_maps(const void* buf, const Grid& g, int tile, int fp16, void* load_map, void* store_map);
 int tma_tile_count();
-int tma_default_tile(int noise_mode, int fp16);
+int tma_default_tile(int noise_mode, int fp16, const Grid& g);
 size_t tensor_map_bytes();
 // many steps of a small FP32 lattice in one launch (lb_step_resident.cu)
 bool resident_fits(const Grid& g);

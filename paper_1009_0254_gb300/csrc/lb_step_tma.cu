@@ -36,6 +36,7 @@
 // error word, gives its loads in flight a bounded chance to land, and returns.
 #include <cuda.h>
 
+#include "lb_limits.cuh"
 #include "lb_pair.cuh"
 
 namespace lbf {
@@ -179,9 +180,13 @@ int tma_tile_count() { return 5; }
 // (shape 4: their exchange stays within a thread for half the rows).  2048^2 and 3000^2 agree; below
 // 512^2 a step is bound by its launch and the shape does not matter.  FP16 (lb_step_half.cu): the shapes
 // its recorded states were computed with, the fastest of that kernel.
-int tma_default_tile(int noise_mode, int fp16) {
+int tma_default_tile(int noise_mode, int fp16, const Grid& g) {
     static const int best[2][5] = {{2, 2, 2, 4, 2}, {4, 1, 3, 0, 1}};
     const int m = noise_mode < 0 ? 0 : (noise_mode > 4 ? 4 : noise_mode);
+    // real space, up to four CTAs a SM of 256 threads: one row of pairs a thread instead of two shortens the
+    // step, which is a tile's latency there (33 x 47 9.7 us against 11.7, 128^2 8.7 and 10.0, 512^2 12.6 and
+    // 13.6; 700^2 16.3 and 16.4, 1000 x 600 19.9 and 18.9)
+    if (!fp16 && m == 3 && (long long)((g.nx + 31) / 32) * ((g.ny + 15) / 16) <= 4LL * device_sms()) return 0;
     return best[fp16 ? 1 : 0][m];
 }
 
@@ -241,12 +246,12 @@ static cudaError_t launch_mode(const void* const map[2], const TmaArgs& ta, int 
 }
 
 // the double-well equation of state, FP32 storage: the default tile of each noise mode
-// (tma_default_tile(noise_mode, 0); the caller encodes the tensor maps for it)
-static cudaError_t launch_poly(const void* const map[2], const TmaArgs& ta, int noise_mode, cudaStream_t s) {
+// (tma_default_tile; the caller encodes the tensor maps for it)
+static cudaError_t launch_poly(const void* const map[2], const TmaArgs& ta, int noise_mode, int tile, cudaStream_t s) {
     switch (noise_mode) {
         case 0: return launch_cfg<64, 8, 256, 0, true>(map, ta, s);
         case 1: return launch_cfg<64, 8, 256, 1, true>(map, ta, s);
-        case 3: return launch_cfg<32, 16, 128, 3, true>(map, ta, s);
+        case 3: return tile == 0 ? launch_cfg<32, 16, 256, 3, true>(map, ta, s) : launch_cfg<32, 16, 128, 3, true>(map, ta, s);
         case 4: return launch_cfg<64, 8, 256, 4, true>(map, ta, s);
         default: return launch_cfg<64, 8, 256, 2, true>(map, ta, s);
     }
@@ -269,7 +274,7 @@ cudaError_t launch_step_tma(const StepArgs& a, const StepArgsD& d, const void* s
     ta.t_hi = a.t_hi;
     ta.rk = a.rk;
     const void* const map[2] = {src_map, dst_map};
-    if (poly) return launch_poly(map, ta, noise_mode, s);
+    if (poly) return launch_poly(map, ta, noise_mode, tile, s);
     switch (noise_mode) {
         case 0: return launch_mode<0>(map, ta, tile, s);
         case 1: return launch_mode<1>(map, ta, tile, s);
