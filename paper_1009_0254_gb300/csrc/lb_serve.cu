@@ -368,7 +368,7 @@ struct lb_server {
     int device = 0;
     size_t budget = 0, in_use = 0, peak = 0;
     int max_slots = 0, max_chunk = 0, grid = 0, grid_rs = 0;
-    cudaStream_t stream = nullptr;
+    cudaStream_t stream = nullptr;           // the worker thread's alone, until the server is destroyed
     cudaStream_t fetch_stream = nullptr;     // reads back kept states (any API thread)
     cudaMemPool_t pool = nullptr;
     // device tables
@@ -405,7 +405,6 @@ struct lb_server {
     bool chunk_pending[2] = {false, false};
     // shared with the API threads
     std::mutex mu;
-    std::mutex gpu;                   // held while issuing GPU work on `stream`
     std::condition_variable cv, cv_done;
     std::deque<Pending> queue;
     std::vector<lb_result> results;   // completed, not yet polled
@@ -506,13 +505,10 @@ bool apply_cancellations(lb_server* s) {
     for (int64_t id : ids) {
         for (auto it = s->running.begin(); it != s->running.end(); ++it) {
             if (it->id != id) continue;
-            {
-                // the slot's staging copies and the chunks in flight must be done before
-                // the slot can be handed to another request (a rare path: synchronise)
-                std::lock_guard<std::mutex> gl(s->gpu);
-                SCK(s, cudaFreeAsync(it->mem, s->stream));
-                SCK(s, cudaStreamSynchronize(s->stream));
-            }
+            // the slot's staging copies and the chunks in flight must be done before
+            // the slot can be handed to another request (a rare path: synchronise)
+            SCK(s, cudaFreeAsync(it->mem, s->stream));
+            SCK(s, cudaStreamSynchronize(s->stream));
             finish_unrun(s, *it, LB_ECANCELED);
             s->running.erase(it);
             break;
@@ -573,7 +569,6 @@ bool admit(lb_server* s) {
         }
     }
     if (take.empty()) return true;
-    std::lock_guard<std::mutex> gl(s->gpu);
     for (size_t q = 0; q < take.size(); ++q) {
         const Pending& pr = take[q];
         Running run;
@@ -754,7 +749,6 @@ bool issue_chunk(lb_server* s) {
             off += (int)kv.second.size();
         }
     }
-    std::lock_guard<std::mutex> gl(s->gpu);
     SCK(s, cudaMemcpyAsync(s->d_active[c], act, n * sizeof(int), cudaMemcpyHostToDevice, s->stream));
     SCK(s, cudaMemcpyAsync(s->d_tb[c], tb, (n + 1) * sizeof(int), cudaMemcpyHostToDevice, s->stream));
     if (!groups.empty()) {
@@ -936,7 +930,6 @@ int lb_server_create(size_t hbm_budget_bytes, int max_active, int max_chunk_step
     if ((e = cudaMemset(s->d_k, 0, sizeof(long long))) != cudaSuccess) return fail_create(e);
     if ((e = cudaMemset(s->d_done, 0, sizeof(unsigned int))) != cudaSuccess) return fail_create(e);
     if ((e = cudaMemset(s->d_err, 0, sizeof(int))) != cudaSuccess) return fail_create(e);
-    using TT = TmaTile<SV_TX, SV_TY>;
     auto kern = step_serve_kernel<SV_TX, SV_TY, SV_NT, false>;
     auto kern_rs = step_serve_kernel<SV_TX, SV_TY, SV_NT, true>;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, serve_smem<false>())) != cudaSuccess)
