@@ -163,8 +163,9 @@ cudaError_t launch_noise49(float2* buf, float2* scratch, const NoiseGenArgs& ga,
     // synthesise xi(k) column block by column block and transform back along y, then along
     // x with the unitary n^-1/2 into buf; the paired blocks need an even width (ny <= 8192).
     // Rows of 256 points and more go through the column-permuted scratch (whole 32-byte
-    // sectors per write, rows gathered back in the first stage of the row transform:
-    // 219 -> 171 us at 4096^2, 118 -> 115 us a step at 2048^2); shorter rows stay in place.
+    // sectors per write from strips of 4 on, halves of one at 256 points, whose strips are
+    // of 2; rows gathered back in the first stage of the row transform: 219 -> 171 us at
+    // 4096^2, 118 -> 115 us a step at 2048^2); shorter rows stay in place.
     const int c = noise_strip(ga.nx, col_strip(ga.nx, ga.ny));
     if (c < 2) return cudaErrorInvalidValue;
     const size_t smem = fft_smem_bytes(ga.ny, c);
@@ -190,7 +191,9 @@ cudaError_t launch_noise49_d(double2* buf, const NoiseGenArgsD& ga, const double
                              cudaStream_t s) {
     const int c = noise_strip(ga.nx, noise_strip_d(ga.nx, ga.ny));
     if (c < 2) return cudaErrorInvalidValue;
-    // a thread per radix-4 butterfly or per pair of wavevectors, whichever is more (both at most 512)
+    // a thread per radix-4 butterfly or per pair of wavevectors, whichever is more, up to the 512 of the
+    // launch bounds (512^2 has 1,024 pairs a CTA, rows of 4,096 points 1,024 butterflies): the pairs are
+    // taken in turns, and a stage takes up to four butterflies a thread, so n count / 16 threads must do
     auto threads = [](int n) { return n < 32 ? 32 : (n > 512 ? 512 : n); };
     const cudaError_t e = launch_fft<noise_cols_kernel_d>(ga.nx / c, threads(ga.ny * c / 2),
                                                           fft_smem_bytes(ga.ny, c, 16), s, buf, ga, c, twy);
