@@ -12,8 +12,8 @@
 //   * rows of a thread's pairs are adjacent, so the density rows of its stencils are loaded once
 //     (12 shared loads for 2 x 2 nodes instead of 36) and their sums over x are shared;
 //   * planes with c_x = 0, the density and all stores move 8 bytes at a time;
-//   * the relaxation and noise factors carry the 1/N_a and w_i of the back-transform (host side,
-//     PairCoef), and the stencil weights 1/6 and 1/12 are folded into kappa;
+//   * the relaxation and noise factors carry the 1/N_a of the back-transform (host side, PairCoef),
+//     and the stencil weights 1/6 and 1/12 are folded into kappa;
 //   * log2, sine and cosine are the flush-to-zero forms (their arguments are never subnormal),
 //     sqrt(2 ln 2) and the sign of the Box-Muller angle's shift are in the noise factors, and
 //     -log2 u1 needs no clamp: u1 <= 1 - 2^-21, so log2 u1 <= -6.8e-7, further from zero than
@@ -65,8 +65,11 @@ __device__ __forceinline__ float sin_ftz(float x) {
 
 // The Box-Muller pairs of two Philox words (gauss_pair of lb_internal.cuh) over
 // GAUSS_SCALE = -sqrt(2 ln 2), which is left to the factors that multiply the normals: the sign of
-// the angle's shift by pi, and the 2 ln 2 of -2 ln u = 2 ln 2 (-log2 u).
-constexpr double GAUSS_SCALE = -1.17741002251547469101;
+// the angle's shift by pi, and the 2 ln 2 of -2 ln u = 2 ln 2 (-log2 u).  The approximations make the
+// normals 1.22e-7 of themselves too small on average (2^31 draws against the FP64 pair), more than half of
+// their error of 2.1e-7; the factors give it back.  Error of a step against FP64, 512^2 real-space noise:
+// 1.84e-7 without this, 1.55e-7 with it (1.74e-7 with scalar nodes).
+constexpr double GAUSS_SCALE = -1.17741002251547469101 * (1.0 + 1.22e-7);
 __device__ __forceinline__ void gauss2(uint32_t wa, uint32_t wb, F2* n0, F2* n1) {
     const F2 u = add2(make_float2(__uint_as_float(((wa >> 9) & 0x7ffff8u) | 0x3f800004u),
                                   __uint_as_float(((wb >> 9) & 0x7ffff8u) | 0x3f800004u)), bc(-1.0f));
@@ -80,30 +83,27 @@ __device__ __forceinline__ void gauss2(uint32_t wa, uint32_t wb, F2* n0, F2* n1)
 
 // --- coefficients ----------------------------------------------------------------------------
 
-// One lattice's coefficients as collide_pair takes them, with c = 1/36 (the diagonal weight; the
-// axis and rest weights are 4 c and 16 c).  A mode's increment enters the back-transform as
-// c D_a / N_a times the common factors 1 (a = 4), 1 (5), 1 (6), 1 (7, 8), 1 (9) of collide_node's
-// d4..d9; noise factors carry GAUSS_SCALE as well (G below).
-constexpr double PAIR_SCALE = 1.0 / 36.0;
-
+// One lattice's coefficients as collide_pair takes them: a mode's rate and noise factors carry the
+// 1 / N_a of its increment in the back-transform (collide_node's d4..d9), noise factors GAUSS_SCALE as
+// well (G below).  The weights w_i stay out of them, so that a rate of -1 is exact: with 1/36 in it a
+// ghost mode kept 3e-8 of itself, and a two-phase run was 6 % further from FP64.
 struct PairCoef {
     float rho0, cs2m;
     float kl, kg;                    // -kappa / 6 and kappa / 144
-    float lb, ls5, ls6, lq, le;      // c (lambda_b / 4, 9 lambda_s / 4, 9 lambda_s, 3 lambda_q / 2, lambda_e / 16)
-    float L44, L49, L94, L99;        // G c (L44, L49) / 4 and G c (L94, L99) / 16
-    float s5, s6, s7;                // G c (9 s5 / 4, 9 s6, 3 s7 / 2)
-    float x4, x9;                    // c / 4 and c / 16: factors of a given (xi_4, xi_9)
+    float lb, ls5, ls6, lq, le;      // lambda_b / 4, 9 lambda_s / 4, 9 lambda_s, 3 lambda_q / 2, lambda_e / 16
+    float L44, L49, L94, L99;        // G (L44, L49) / 4 and G (L94, L99) / 16
+    float s5, s6, s7;                // G (9 s5 / 4, 9 s6, 3 s7 / 2)
 };
 
 // the double well's pressure and the noise at the local density (single lattices)
 struct PairLocal {
     float e2, e3, e4;
     float cq[4];
-    float lu[9];                     // of x44 c^2 / 16, x49 c^2 / 64, x99 c^2 / 256 per unit density, then
-                                     // G c (9 / 4, 9, 3 / 2) times the roots of x55, x66, x77
+    float lu[9];                     // of x44 / 16, x49 / 64, x99 / 256 per unit density, then
+                                     // G (9 / 4, 9, 3 / 2) times the roots of x55, x66, x77
 };
 
-// real-space correlated noise: G c / 4 and G c / 16 times the factors / 4 of Xi at k^2 = 0, 4, 16/3
+// real-space correlated noise: G / 4 and G / 16 times the factors / 4 of Xi at k^2 = 0, 4, 16/3
 struct PairStencil {
     float sL[3][4];
 };
@@ -111,17 +111,16 @@ struct PairStencil {
 template <typename S>
 __host__ inline void pair_coef(double rho0, double cs2m, double kappa, double lb, double ls, double lq, double le,
                                const S L[4], const S s[3], PairCoef* o) {
-    const double c = PAIR_SCALE;
     o->rho0 = (float)rho0;
     o->cs2m = (float)cs2m;
     o->kl = (float)(-kappa / 6.0);
     o->kg = (float)(kappa / 144.0);
-    o->lb = (float)(c * lb / 4.0);
-    o->ls5 = (float)(c * ls * 2.25);
-    o->ls6 = (float)(c * ls * 9.0);
-    o->lq = (float)(c * lq * 1.5);
-    o->le = (float)(c * le / 16.0);
-    const double G = GAUSS_SCALE * c;
+    o->lb = (float)(lb / 4.0);
+    o->ls5 = (float)(ls * 2.25);
+    o->ls6 = (float)(ls * 9.0);
+    o->lq = (float)(lq * 1.5);
+    o->le = (float)(le / 16.0);
+    const double G = GAUSS_SCALE;
     o->L44 = (float)(G * L[0] / 4.0);
     o->L49 = (float)(G * L[1] / 4.0);
     o->L94 = (float)(G * L[2] / 16.0);
@@ -129,13 +128,11 @@ __host__ inline void pair_coef(double rho0, double cs2m, double kappa, double lb
     o->s5 = (float)(G * s[0] * 2.25);
     o->s6 = (float)(G * s[1] * 9.0);
     o->s7 = (float)(G * s[2] * 1.5);
-    o->x4 = (float)(c / 4.0);
-    o->x9 = (float)(c / 16.0);
 }
 
 template <typename S>
 __host__ inline void pair_stencil(const S sL[3][4], PairStencil* o) {
-    const double G = GAUSS_SCALE * PAIR_SCALE;
+    const double G = GAUSS_SCALE;
     for (int j = 0; j < 3; ++j) {
         o->sL[j][0] = (float)(G * sL[j][0] / 4.0);
         o->sL[j][1] = (float)(G * sL[j][1] / 4.0);
@@ -146,13 +143,12 @@ __host__ inline void pair_stencil(const S sL[3][4], PairStencil* o) {
 
 template <typename S>
 __host__ inline void pair_local(double e2, double e3, double e4, const S cq[4], const S lu[9], PairLocal* o) {
-    const double c = PAIR_SCALE;
     o->e2 = (float)e2;
     o->e3 = (float)e3;
     o->e4 = (float)e4;
     for (int q = 0; q < 4; ++q) o->cq[q] = (float)cq[q];
-    const double f[9] = {c * c / 16.0, c * c / 16.0, c * c / 64.0, c * c / 64.0, c * c / 256.0, c * c / 256.0,
-                         GAUSS_SCALE * c * 2.25, GAUSS_SCALE * c * 9.0, GAUSS_SCALE * c * 1.5};
+    const double f[9] = {1 / 16.0, 1 / 16.0, 1 / 64.0, 1 / 64.0, 1 / 256.0, 1 / 256.0,
+                         GAUSS_SCALE * 2.25, GAUSS_SCALE * 9.0, GAUSS_SCALE * 1.5};
     for (int q = 0; q < 9; ++q) o->lu[q] = (float)(f[q] * lu[q]);
 }
 
@@ -282,15 +278,16 @@ __device__ __forceinline__ void collide_pair(const Args& a, const PairLocal* loc
     const F2 e4 = mul2(fma2(d9, bc(2.0f), d4), bc(4.0f));
     const F2 D1 = add2(e4, d6), D2 = sub2(e4, d6);
     const F2 p = add2(d7, d8), m = sub2(d7, d8);
-    o[5] = add2(f[5], fma2(p, bc(2.0f), D1));
-    o[7] = add2(f[7], fma2(p, bc(-2.0f), D1));
-    o[6] = add2(f[6], fma2(m, bc(-2.0f), D2));
-    o[8] = add2(f[8], fma2(m, bc(2.0f), D2));
-    o[0] = fma2(sub2(d9, d4), bc(32.0f), f[0]);
-    o[1] = fma2(sub2(A1, d7), bc(4.0f), f[1]);
-    o[2] = fma2(sub2(A2, d8), bc(4.0f), f[2]);
-    o[3] = fma2(add2(A1, d7), bc(4.0f), f[3]);
-    o[4] = fma2(add2(A2, d8), bc(4.0f), f[4]);
+    const F2 u0 = bc(8.0f / 9.0f), u1 = bc(1.0f / 9.0f), u5 = bc(1.0f / 36.0f);
+    o[5] = fma2(fma2(p, bc(2.0f), D1), u5, f[5]);
+    o[7] = fma2(fma2(p, bc(-2.0f), D1), u5, f[7]);
+    o[6] = fma2(fma2(m, bc(-2.0f), D2), u5, f[6]);
+    o[8] = fma2(fma2(m, bc(2.0f), D2), u5, f[8]);
+    o[0] = fma2(sub2(d9, d4), u0, f[0]);
+    o[1] = fma2(sub2(A1, d7), u1, f[1]);
+    o[2] = fma2(sub2(A2, d8), u1, f[2]);
+    o[3] = fma2(add2(A1, d7), u1, f[3]);
+    o[4] = fma2(add2(A2, d8), u1, f[4]);
 }
 
 // --- a staged tile ------------------------------------------------------------------------------
@@ -562,8 +559,8 @@ __device__ __forceinline__ void tile_collide(const Args& a, const PairLocal* loc
         F2 v4 = bc(0.f), v9 = bc(0.f);
         if constexpr (MODE == 2) {
             const float4 v = *reinterpret_cast<const float4*>(xi49 + (long long)y * g.nx + x);
-            v4 = mul2(make_float2(v.x, v.z), bc(a.x4));
-            v9 = mul2(make_float2(v.y, v.w), bc(a.x9));
+            v4 = mul2(make_float2(v.x, v.z), bc(0.25f));
+            v9 = mul2(make_float2(v.y, v.w), bc(0.0625f));
         }
         if constexpr (MODE == 3) {
             const F2 e = reinterpret_cast<const F2*>(xch + ST::ER)[(ly + j) * ST::W + p];
