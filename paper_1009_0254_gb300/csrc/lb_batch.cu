@@ -88,7 +88,8 @@ __device__ __forceinline__ TilePos locate(const EnsParams& p, int tile) {
 // The engine's step is the single-lattice kernel's (lb_step_tma.cu, lb_pair.cuh) plus, per tile, its
 // position and its replica's record; both bound it beside DRAM (252 to 297 instructions a node against
 // 209 and up).  512 replicas of 32^2 to 256^2, best tile: 188 us a step with scalar nodes and two
-// stages, 164 in this form; real-space correlated noise 333 and 228; 16 replicas of 1024^2 258 and 222.
+// stages, 164 in this form (163 with the spectra of every 100th step since the record is copied as
+// in lb_ens.cuh); real-space correlated noise 333 and 228; 16 replicas of 1024^2 258 and 222.
 // RS: the variant that also steps replicas with real-space correlated noise (its extra path
 // raises the register count, so launches without such replicas use the lean variant)
 template <int TX, int TY, int NT, bool RS>

@@ -10,7 +10,7 @@
 // 4096^2 182 instead of 222, with other roundings; the pairs' data movement around collide_node took 207 and
 // had other roundings too, as the compiler fuses the same source otherwise in another kernel.
 //
-// What bounds it: issue (375 instructions a node, FP32 arithmetic on half the bytes).  4096^2, us a step: no
+// What bounds it: issue (368 instructions a node at 71 % issue, FP32 arithmetic on half the bytes).  4096^2, us a step: no
 // noise 162, uncorrelated 222, k-space correlated 228 (the step kernel), real space 339, local density 233.
 #include <cuda.h>
 
